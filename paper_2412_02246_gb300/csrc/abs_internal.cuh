@@ -41,12 +41,17 @@ struct Setup {
     // device copies (owned by the context)
     int64_t *d_q = nullptr;
     int64_t *d_lat_off = nullptr;
-    int64_t *d_ring_off = nullptr;  // [3][nb+1] family f, ring m: f * up_off[nb] + up_off[m]
     int32_t *d_ijk = nullptr;
     float4 *d_tw = nullptr;       // exp(-2 pi i t / N) = c + i s, t < N, as packed double-float pairs:
                                   // [2t] = (c.hi, c.hi, c.lo, c.lo), [2t+1] = (-s.hi, s.hi, -s.lo, s.lo),
                                   // then in FP32: [2N + t] = (c, c, -s, s)
     int32_t *d_Rm = nullptr;
+    // the rings' cell lists, orbits and byte map (counts.cu), one allocation with its parts at rg_at,
+    // and the largest numbers of work items the counts can cut
+    void *d_ring_geom = nullptr;
+    size_t rg_at[7] = {0, 0, 0, 0, 0, 0, 0};
+    int n_orb = 0;
+    int item_cap[2] = {0, 0};
     // ordered closed-triangle counts of the full annuli [nb][nb][nb] (halved),
     // a property of the ring geometry, computed on first use
     unsigned long long *d_full_counts = nullptr;
@@ -228,6 +233,8 @@ abs_status launch_triple_sums(abs_ctx *ctx, const Setup &s, const float *d_field
 // the fields already.
 abs_status launch_triple_tc(abs_ctx *ctx, const Setup &s, const float *d_fields,
                             int32_t n_trip, const int32_t *d_ijk, double *d_sum);
+// Uploads the ring geometry of a derived setup (d_ring_geom); false if it cannot be allocated.
+bool make_ring_geometry(Setup &s);
 // Ring tables (cell lists, byte map) from d_mask, or, with d_accw given, from
 // the FP64 weight sums before the mirror (a cell is filled when it or its
 // mirror has a nonzero sum), then exact counts (d_count may be NULL) and, if

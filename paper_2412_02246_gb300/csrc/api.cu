@@ -305,8 +305,8 @@ static T *upload(const std::vector<T> &v) {
 static void free_setup(Setup &s) {
     cudaFree(s.d_q);
     cudaFree(s.d_lat_off);
-    cudaFree(s.d_ring_off);
-    s.d_ring_off = nullptr;
+    cudaFree(s.d_ring_geom);
+    s.d_ring_geom = nullptr;
     cudaFree(s.d_ijk);
     cudaFree(s.d_tw);
     cudaFree(s.d_Rm);
@@ -354,16 +354,10 @@ const Setup *get_setup(abs_ctx *ctx, const abs_config *cfg, abs_status &st) {
     }
     s->d_q = upload(s->q);
     s->d_lat_off = upload(s->lat_off);
-    {
-        std::vector<int64_t> ro(3 * (size_t)(s->nb + 1));
-        for (int f = 0; f < 3; ++f)
-            for (int m = 0; m <= s->nb; ++m) ro[(size_t)f * (s->nb + 1) + m] = f * s->up_off[s->nb] + s->up_off[m];
-        s->d_ring_off = upload(ro);
-    }
     s->d_ijk = upload(s->ijk);
     s->d_tw = upload(tw);
     s->d_Rm = upload(std::vector<int32_t>(s->Rm.begin(), s->Rm.end()));
-    if (!s->d_q || !s->d_lat_off || !s->d_ring_off || !s->d_ijk || !s->d_tw || !s->d_Rm) {
+    if (!make_ring_geometry(*s) || !s->d_q || !s->d_lat_off || !s->d_ijk || !s->d_tw || !s->d_Rm) {
         free_setup(*s);
         st = fail(ctx, ABS_ERR_OOM, "setup tables");
         return nullptr;
