@@ -6,22 +6,27 @@
 //   V(U) = sum over pixels of dtheta^2 A(theta) T(theta) exp(+i 2 pi U.theta),
 //   pixel (row b, column a) at theta = ((a - m/2) dtheta, (b - m/2) dtheta).
 //
-// One thread per visibility; the weighted map is staged through shared memory
-// in tiles that every thread of the block walks in the same order.  The phase
-// U.theta (hundreds of cycles for baselines of hundreds of wavelengths over a
-// radian) is carried as a double-float pair and reduced to its fractional
-// cycle before the FP32 sine and cosine (the SFU's), at the start of every run
-// of 16 pixels of a row; the run's other terms are rotated by one column's
-// phase (sine and cosine to a few ulp).
-// The FP32 terms are folded into double-float sums every 64 pixels.
+// The phase separates, exp(i 2 pi U.theta) = exp(i 2 pi u theta_x) exp(i 2 pi v theta_y), so
+// every visibility's sum is a product of matrices: per row b of the map the real-by-complex
+// product R[b] = sum_a W[b][a] exp(i 2 pi u theta_a), two multiply-adds a term, then
+// V = sum_b exp(i 2 pi v theta_b) R[b].  A thread owns two visibilities and SIM_A columns whose
+// column phases it keeps in registers while it walks the rows (k_dft); the column blocks and
+// the row ranges are spread over CTAs and their partial sums added in a fixed order
+// (k_dft_reduce).  The phases (hundreds of cycles for baselines of hundreds of wavelengths
+// over a radian) are carried as double-float pairs and reduced to their fractional cycle
+// before the FP32 sine and cosine.
+#include <algorithm>
+
 #include "abs_internal.cuh"
 
 namespace absk {
 namespace {
 
-constexpr int SIM_T = 256;       // visibilities per CTA
-constexpr int SIM_TILE = 4096;   // map pixels staged per pass
-constexpr int SIM_FOLD = 64;     // pixels summed in FP32 before each double-float fold
+constexpr int SIM_T = 128;       // threads per CTA
+constexpr int SIM_V = 2;         // visibilities of a thread
+constexpr int SIM_A = 32;        // map columns of a thread (their phases: 2 x SIM_A x SIM_V registers)
+constexpr int SIM_R = 4;         // map rows walked together
+constexpr int SIM_ROWS = 32;     // map rows staged in shared memory per pass
 
 __global__ void k_sky_weights(int m, double dth, const float *__restrict__ sky, int beam, double bp,
                               float *__restrict__ W) {
@@ -60,74 +65,144 @@ __device__ __forceinline__ void df_scale(float h, float l, float k, float &zh, f
     zl = __fsub_rn(t, __fsub_rn(zh, p));
 }
 
-// exp(i 2 pi phi) for a double-float phase phi in cycles, from its fractional cycle f
-// (|f| <= 1/2).  fast: the SFU's __sincosf of 2 pi f (absolute error about 4e-7 over
-// [-pi, pi]); else sincospif (a few ulp, but slow here: it keeps the FP64 pipe busy).
-__device__ __forceinline__ float2 cis_cycles(float h, float l, bool fast) {
+// exp(i 2 pi phi) for a double-float phase phi in cycles: the fractional cycle f, |f| <= 1/2,
+// to the nearest quarter turn q and the rest r, |r| <= 1/8, then the Taylor series of sine and
+// cosine on |2 pi r| <= pi / 4 (truncation below 2e-9) turned by q quarters.  About 1e-7 at
+// most, without the FP64 pipe sincospif keeps busy here or the 4e-7 of the SFU's __sincosf.
+__device__ __forceinline__ float2 cis_cycles(float h, float l) {
     const float f = __fadd_rn(__fsub_rn(h, rintf(h)), l);
-    float s, c;
-    if (fast) __sincosf(6.28318531f * f, &s, &c);
-    else sincospif(2.0f * f, &s, &c);
-    return make_float2(c, s);
+    const float qf = rintf(4.0f * f);
+    const float t = 6.28318531f * fmaf(-0.25f, qf, f), t2 = t * t;
+    float s = fmaf(t2, 2.75573192e-6f, -1.98412698e-4f);
+    s = fmaf(t2, s, 8.33333333e-3f);
+    s = fmaf(t2, s, -1.66666667e-1f);
+    s = fmaf(t * t2, s, t);
+    float c = fmaf(t2, -2.75573192e-7f, 2.48015873e-5f);
+    c = fmaf(t2, c, -1.38888889e-3f);
+    c = fmaf(t2, c, 4.16666667e-2f);
+    c = fmaf(t2, c, -0.5f);
+    c = fmaf(t2, c, 1.0f);
+    const int q = (int)qf;
+    const float a = (q & 1) ? s : c, b = (q & 1) ? c : s;   // |cos|, |sin| after the quarter turns
+    return make_float2(((q + 1) & 2) ? -a : a, (q & 2) ? -b : b);
 }
 
-// The phase u theta_x(a) + v theta_y(b) in cycles is exact (double-float) at the
-// first pixel of every run of SIM_RUN in a row; in between, the term is rotated
-// by exp(i 2 pi u dtheta) (a complex multiply), so a run's rounding drift is a
-// few units in the last place.
-constexpr int SIM_RUN = 16;
+// k (h, l) cycles for an integer k, |k| <= 8192.
+__device__ __forceinline__ float2 cis_multiple(float h, float l, int k) {
+    float zh, zl;
+    df_scale(h, l, (float)k, zh, zl);
+    return cis_cycles(zh, zl);
+}
 
+__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
+    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+}
+
+// SIM_V visibilities a thread, SIM_A columns from blockIdx.y SIM_A, rows [blockIdx.z rows_per, + rows_per):
+// their sums over them as double-float pairs (re.hi, re.lo, im.hi, im.lo) in part[z gridDim.y + y][vis].
+// Bound by FP32 multiply-adds: per term one half of a packed FFMA2 for each of re and im; one map load
+// (LDS.128, a broadcast) serves four FFMA2 of each visibility.  The columns' FP32 sums run in chains of
+// SIM_A / 2 terms, eight rows' terms are added in FP32 and everything beyond in double-float; a row
+// phase is rotated from the one SIM_R rows before, at most SIM_ROWS / SIM_R times from an exact one.
 __global__ void __launch_bounds__(SIM_T) k_dft(int m, double dth, const float *__restrict__ W, int64_t n_vis,
-                                               const float2 *__restrict__ uv, float2 *__restrict__ vis) {
-    __shared__ float ws[SIM_TILE];
-    const int64_t e = (int64_t)blockIdx.x * SIM_T + threadIdx.x;
-    const bool on = e < n_vis;
-    const float2 U = on ? uv[e] : make_float2(0.f, 0.f);
-    // u dtheta and v dtheta as double-float pairs (from the FP64 products), and the phase
-    // of pixel (0, 0): (u + v) theta_0
-    const double th0 = -(double)(m / 2) * dth;
-    const double cu = (double)U.x * dth, cv = (double)U.y * dth, c0 = ((double)U.x + (double)U.y) * th0;
-    const float cuh = (float)cu, cul = (float)(cu - (double)cuh);
-    const float cvh = (float)cv, cvl = (float)(cv - (double)cvh);
-    float rh = (float)c0, rl = (float)(c0 - (double)rh);   // the row's phase at a = 0
-    const float2 w = cis_cycles(cuh, cul, false);          // one column's rotation (accurate: it compounds)
-    const int64_t npix = (int64_t)m * m;
-    float reh = 0.f, rel = 0.f, imh = 0.f, iml = 0.f;   // double-float sums of the folded blocks
-    float fr = 0.f, fi = 0.f;
-    float2 z = make_float2(1.f, 0.f);
-    int a = 0, nf = 0;
-    for (int64_t p0 = 0; p0 < npix; p0 += SIM_TILE) {
-        const int np = (int)min((int64_t)SIM_TILE, npix - p0);
+                                               const float2 *__restrict__ uv, int rows_per,
+                                               float4 *__restrict__ part) {
+    __shared__ __align__(16) float ws[SIM_ROWS][SIM_A];
+    const int64_t e = (int64_t)blockIdx.x * (SIM_T * SIM_V) + threadIdx.x;
+    const int a0 = blockIdx.y * SIM_A, b0 = blockIdx.z * rows_per, b1 = min(m, b0 + rows_per);
+    float cvh[SIM_V], cvl[SIM_V];                    // v dtheta in cycles as a double-float pair (from the FP64 product)
+    float2 xr[SIM_V][SIM_A / 2], xi[SIM_V][SIM_A / 2];   // the columns' phases, two neighbours to a pair
+    float2 turn[SIM_V][SIM_R];                       // one to SIM_R rows further
+#pragma unroll
+    for (int n = 0; n < SIM_V; ++n) {
+        const int64_t en = e + n * SIM_T;
+        const float2 U = en < n_vis ? uv[en] : make_float2(0.f, 0.f);
+        const double cu = (double)U.x * dth, cv = (double)U.y * dth;
+        const float cuh = (float)cu, cul = (float)(cu - (double)cuh);
+        cvh[n] = (float)cv;
+        cvl[n] = (float)(cv - (double)cvh[n]);
+#pragma unroll
+        for (int k = 0; k < SIM_A / 2; ++k) {
+            const float2 p = cis_multiple(cuh, cul, a0 + 2 * k - m / 2), q = cis_multiple(cuh, cul, a0 + 2 * k + 1 - m / 2);
+            xr[n][k] = make_float2(p.x, q.x);
+            xi[n][k] = make_float2(p.y, q.y);
+        }
+#pragma unroll
+        for (int r = 0; r < SIM_R; ++r) turn[n][r] = cis_multiple(cvh[n], cvl[n], r + 1);
+    }
+    float reh[SIM_V] = {}, rel[SIM_V] = {}, imh[SIM_V] = {}, iml[SIM_V] = {};
+    for (int r0 = b0; r0 < b1; r0 += SIM_ROWS) {
+        const int nr = min(SIM_ROWS, b1 - r0);
         __syncthreads();
-        for (int i = threadIdx.x; i < np; i += SIM_T) ws[i] = W[p0 + i];
+        for (int i = threadIdx.x; i < SIM_ROWS * SIM_A; i += SIM_T) {   // zeros past the map and the range
+            const int r = i / SIM_A, a = i % SIM_A;
+            ws[r][a] = r < nr && a0 + a < m ? W[(int64_t)(r0 + r) * m + a0 + a] : 0.f;
+        }
         __syncthreads();
-        for (int i = 0; i < np; ++i) {
-            if (a % SIM_RUN == 0) {
-                float ph, pl, qh, ql;
-                df_scale(cuh, cul, (float)a, ph, pl);
-                df_add(rh, rl, ph, pl, qh, ql);
-                z = cis_cycles(qh, ql, true);
-            } else {
-                z = make_float2(fmaf(z.x, w.x, -z.y * w.y), fmaf(z.x, w.y, z.y * w.x));
+        float2 y[SIM_V], v[SIM_V];   // the phase of the first of SIM_R rows; the FP32 sum of up to 2 SIM_R rows
+#pragma unroll
+        for (int n = 0; n < SIM_V; ++n) {
+            y[n] = cis_multiple(cvh[n], cvl[n], r0 - m / 2);
+            v[n] = make_float2(0.f, 0.f);
+        }
+        for (int r = 0; r < nr; r += SIM_R) {
+            float2 sr[SIM_V][SIM_R], si[SIM_V][SIM_R];
+#pragma unroll
+            for (int n = 0; n < SIM_V; ++n)
+#pragma unroll
+                for (int q = 0; q < SIM_R; ++q) sr[n][q] = si[n][q] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < SIM_A / 4; ++k) {
+#pragma unroll
+                for (int q = 0; q < SIM_R; ++q) {
+                    const float4 w = ((const float4 *)ws[r + q])[k];
+#pragma unroll
+                    for (int n = 0; n < SIM_V; ++n) {
+                        sr[n][q] = __ffma2_rn(make_float2(w.x, w.y), xr[n][2 * k], sr[n][q]);
+                        si[n][q] = __ffma2_rn(make_float2(w.x, w.y), xi[n][2 * k], si[n][q]);
+                        sr[n][q] = __ffma2_rn(make_float2(w.z, w.w), xr[n][2 * k + 1], sr[n][q]);
+                        si[n][q] = __ffma2_rn(make_float2(w.z, w.w), xi[n][2 * k + 1], si[n][q]);
+                    }
+                }
             }
-            const float wt = ws[i];
-            fr = fmaf(wt, z.x, fr);
-            fi = fmaf(wt, z.y, fi);
-            if (++nf == SIM_FOLD) {
-                df_add(reh, rel, fr, 0.f, reh, rel);
-                df_add(imh, iml, fi, 0.f, imh, iml);
-                fr = fi = 0.f;
-                nf = 0;
-            }
-            if (++a == m) {
-                a = 0;
-                df_add(rh, rl, cvh, cvl, rh, rl);
+#pragma unroll
+            for (int n = 0; n < SIM_V; ++n) {
+                float2 z = make_float2(sr[n][0].x + sr[n][0].y, si[n][0].x + si[n][0].y);
+#pragma unroll
+                for (int q = 1; q < SIM_R; ++q) {
+                    const float2 t = cmul(turn[n][q - 1], make_float2(sr[n][q].x + sr[n][q].y, si[n][q].x + si[n][q].y));
+                    z = make_float2(z.x + t.x, z.y + t.y);
+                }
+                z = cmul(y[n], z);
+                y[n] = cmul(y[n], turn[n][SIM_R - 1]);
+                v[n] = make_float2(v[n].x + z.x, v[n].y + z.y);
+                if ((r & SIM_R) || r + SIM_R >= nr) {
+                    df_add(reh[n], rel[n], v[n].x, 0.f, reh[n], rel[n]);
+                    df_add(imh[n], iml[n], v[n].y, 0.f, imh[n], iml[n]);
+                    v[n] = make_float2(0.f, 0.f);
+                }
             }
         }
     }
-    df_add(reh, rel, fr, 0.f, reh, rel);
-    df_add(imh, iml, fi, 0.f, imh, iml);
-    if (on) vis[e] = make_float2(__fadd_rn(reh, rel), __fadd_rn(imh, iml));
+#pragma unroll
+    for (int n = 0; n < SIM_V; ++n)
+        if (e + n * SIM_T < n_vis)
+            part[((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * n_vis + e + n * SIM_T] =
+                make_float4(reh[n], rel[n], imh[n], iml[n]);
+}
+
+// The parts of a visibility added in order.
+__global__ void __launch_bounds__(256) k_dft_reduce(int64_t n_vis, int parts, const float4 *__restrict__ part,
+                                                    float2 *__restrict__ vis) {
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n_vis) return;
+    float reh = 0.f, rel = 0.f, imh = 0.f, iml = 0.f;
+    for (int k = 0; k < parts; ++k) {
+        const float4 p = part[k * n_vis + e];
+        df_add(reh, rel, p.x, p.y, reh, rel);
+        df_add(imh, iml, p.z, p.w, imh, iml);
+    }
+    vis[e] = make_float2(__fadd_rn(reh, rel), __fadd_rn(imh, iml));
 }
 
 }  // namespace
@@ -136,12 +211,23 @@ abs_status launch_simulate_vis(abs_ctx *ctx, int32_t m, double dtheta, const flo
                                double beam_param, int64_t n_vis, const float *d_uv, float *d_vis) {
     const int64_t npix = (int64_t)m * m;
     float *W = (float *)workspace(ctx, "sim.weights", sizeof(float) * (size_t)npix);
-    if (!W) return fail(ctx, ABS_ERR_OOM, "simulator workspace");
+    // column blocks and row ranges (whole staged passes) so that the launch holds about eight waves
+    // of CTAs, two to an SM by their registers; the visibilities in slabs whose parts take 256 MB at most
+    const int ny = (int)cdiv(m, SIM_A);
+    const int64_t slab = std::min<int64_t>(n_vis, std::max<int64_t>(SIM_T * SIM_V, (((int64_t)256 << 20) / 16 / ny) / (SIM_T * SIM_V) * (SIM_T * SIM_V)));
+    const int64_t ctas = std::max<int64_t>(cdiv(slab, SIM_T * SIM_V) * ny, 1);
+    const int want = (int)std::min<int64_t>(cdiv(m, SIM_ROWS), cdiv((int64_t)16 * ctx->sm_count, ctas));
+    const int rows_per = (int)cdiv(cdiv(m, want), SIM_ROWS) * SIM_ROWS, nz = (int)cdiv(m, rows_per);
+    float4 *part = (float4 *)workspace(ctx, "sim.parts", sizeof(float4) * (size_t)(ny * nz) * slab);
+    if (!W || !part) return fail(ctx, ABS_ERR_OOM, "simulator workspace");
     StageTimer timer(ctx, "simulate_vis");
     k_sky_weights<<<(unsigned)cdiv(npix, 256), 256, 0, ctx->stream>>>(m, dtheta, d_sky, beam, beam_param, W);
-    if (n_vis > 0)
-        k_dft<<<(unsigned)cdiv(n_vis, SIM_T), SIM_T, 0, ctx->stream>>>(m, dtheta, W, n_vis, (const float2 *)d_uv,
-                                                                       (float2 *)d_vis);
+    for (int64_t v0 = 0; v0 < n_vis; v0 += slab) {
+        const int64_t nv = std::min(slab, n_vis - v0);
+        k_dft<<<dim3((unsigned)cdiv(nv, SIM_T * SIM_V), ny, nz), SIM_T, 0, ctx->stream>>>(m, dtheta, W, nv, (const float2 *)d_uv + v0,
+                                                                                rows_per, part);
+        k_dft_reduce<<<(unsigned)cdiv(nv, 256), 256, 0, ctx->stream>>>(nv, ny * nz, part, (float2 *)d_vis + v0);
+    }
     return check_launch(ctx, "visibility simulator");
 }
 
