@@ -177,8 +177,8 @@ const Setup *get_setup(abs_ctx *ctx, const abs_config *cfg, abs_status &st);
 // cell only (launch_grid_accumulate's estimate form reads it).
 abs_status launch_grid_plan(abs_ctx *ctx, const Setup &s, int64_t n_vis, const float *d_uv,
                             bool rings_only = false);
-// With d_grid == d_wsum == nullptr only the FP64 accumulators (and, if d_mask,
-// the filled mask) are produced.  acc_zeroed: the caller has already cleared
+// With d_grid == d_wsum == nullptr only the FP64 accumulators are produced.
+// acc_zeroed: the caller has already cleared
 // the accumulators (grid_acc_buffers) on this stream's timeline.
 abs_status launch_grid_accumulate(abs_ctx *ctx, const Setup &s, int64_t n_vis, const float *d_vis,
                                   float *d_grid, float *d_wsum, uint8_t *d_mask, bool acc_zeroed = false);
@@ -242,9 +242,6 @@ bool make_ring_geometry(Setup &s);
 abs_status launch_counts(abs_ctx *ctx, const Setup &s, const uint8_t *d_mask, int32_t n_trip,
                          const int32_t *d_ijk, int64_t *d_count, double *d_ellbar,
                          const double *d_accw = nullptr);
-// Exclusive scan of len uint32 values on the context's stream (2 kernels);
-// bsum holds cdiv(len, 4096) + 1 entries.  False if its counter cannot be allocated.
-bool scan_u32(abs_ctx *ctx, const uint32_t *in, int64_t len, uint32_t *out, uint32_t *bsum);
 abs_status launch_normalise(abs_ctx *ctx, const Setup &s, int32_t n_trip, const double *d_sum,
                             const int64_t *d_count, double *d_B);
 // B = Re S / (A S_W) (NaN where S_W = 0), the literal denominator of Eq. estimator_t.

@@ -6,9 +6,9 @@
 // the same sum.
 //
 // Plan (per baseline set): key every visibility by its 16x16-cell uv tile and
-// its cell in the tile, stable-sort by that key (LSD radix, two passes up to
-// about 2040^2 cells, three beyond), and write the sorted positions and
-// original indices; the sorted order is cut into work units of UMAX records.
+// its cell in the tile and stable-sort positions and original indices by that
+// key (LSD radix, two passes up to about 500^2 cells, three beyond); the
+// sorted order is cut into work units of UMAX records.
 //
 // Accumulation (per realisation): one CTA per unit stages the unit in shared
 // memory, forms the 1-D Gaussian weights and cuts it into runs of
@@ -22,6 +22,8 @@
 // division residual) and the exponent argument formed in double-float, so
 // that the only sizeable error is that of expf itself.
 #include <algorithm>
+#include <cmath>
+#include <cstring>
 
 #include "abs_internal.cuh"
 
@@ -35,6 +37,7 @@ constexpr unsigned FULL = 0xffffffffu;
 struct GridGeom {
     int n, half, r, ks, tt, off, kernel;
     float du, inv_du, s_hi, s_lo;
+    bool by_inv;   // quotients by the correctly rounded reciprocal inv_du (see quotient)
 };
 
 // The key space of the plan: every nearest cell whose footprint can reach the grid
@@ -53,101 +56,82 @@ GridGeom geom(const Setup &s, bool rings_only = false) {
     g.off = reach + g.r;
     g.kernel = s.kernel;
     g.du = s.du;
+    // 1 / dU correctly rounded: of the FP32 neighbours of the rounded quotient the one with the smallest
+    // |1 - y dU| (exact in FP64)
     g.inv_du = (float)(1.0 / (double)s.du);
+    for (float y : {std::nextafter(g.inv_du, 0.f), std::nextafter(g.inv_du, INFINITY)})
+        if (std::fabs(1.0 - (double)y * s.du) < std::fabs(1.0 - (double)g.inv_du * s.du)) g.inv_du = y;
+    uint32_t bits;
+    std::memcpy(&bits, &s.du, sizeof bits);
+    g.by_inv = (bits & 0x7fffffu) != 0x7fffffu && s.du > 1e-30f && s.du < 1e30f;
     g.s_hi = s.s_hi;
     g.s_lo = s.s_lo;
     return g;
 }
 
-__device__ __forceinline__ int64_t cell_index(int n, int gx, int gy) {
-    const int ix = gx < 0 ? gx + n : gx;
-    const int iy = gy < 0 ? gy + n : gy;
-    return (int64_t)iy * n + ix;
-}
-
-// exp(-(s_hi + s_lo) (d - f_hi - f_lo)^2) with the argument in double-float.
-__device__ __forceinline__ float wexp(float d, float f_hi, float f_lo, float s_hi, float s_lo) {
-    const float t = __fsub_rn(d, f_hi);                 // TwoSum(d, -f_hi)
-    const float bp = __fsub_rn(t, d);
-    const float e = __fadd_rn(__fsub_rn(d, __fsub_rn(t, bp)), __fsub_rn(-f_hi, bp));
-    const float a_hi = t, a_lo = __fsub_rn(e, f_lo);
-    const float p = __fmul_rn(a_hi, a_hi);
-    const float pe = fmaf(a_hi, a_hi, -p);              // exact square error
-    const float qq = fmaf(2.0f * a_hi, a_lo, pe);
-    const float arg_hi = __fmul_rn(-s_hi, p);
-    const float arg_e = fmaf(-s_hi, p, -arg_hi);        // exact product error
-    const float arg_lo = arg_e - s_hi * qq - s_lo * p;
-    return expf(arg_hi) * (1.0f + arg_lo);
+// exp(-(s_hi + s_lo) (d - f_hi - f_lo)^2) for the x and the y offset of a visibility at once, the
+// argument in double-float (packed FP32x2).  nf = -f_hi, nfl = -f_lo.  The difference t = d - f_hi and
+// its error e are exact: d is an integer and |f_hi| <= |d| unless d = 0 (Fast2Sum).
+__device__ __forceinline__ float2 wexp2(float d, float2 nf, float2 nfl, float s_hi, float s_lo) {
+    const float2 dd = make_float2(d, d), nd = make_float2(-d, -d), f = make_float2(-nf.x, -nf.y);
+    const float2 ns = make_float2(-s_hi, -s_hi), sl = make_float2(s_lo, s_lo);
+    const float2 t = __fadd2_rn(dd, nf), nt = __fadd2_rn(nd, f);   // +-(d - f_hi)
+    const float2 a_lo = __fadd2_rn(__fadd2_rn(__fadd2_rn(dd, nt), nf), nfl);
+    const float2 np = __fmul2_rn(t, nt);                           // -t^2
+    const float2 pe = __ffma2_rn(t, t, np);                        // its error
+    const float2 qq = __ffma2_rn(__fadd2_rn(t, t), a_lo, pe);
+    const float2 narg = __fmul2_rn(ns, np);                        // s_hi t^2 = -arg_hi
+    const float2 arg_e = __ffma2_rn(make_float2(s_hi, s_hi), np, narg);   // error of the product
+    const float2 arg_lo = __ffma2_rn(sl, np, __ffma2_rn(ns, qq, arg_e));
+    const float2 c = __fadd2_rn(make_float2(1.f, 1.f), arg_lo);
+    return __fmul2_rn(make_float2(expf(-narg.x), expf(-narg.y)), c);
 }
 
 // ------------------------------------------------------------------ plan kernels
 // The plan is a stable counting sort of the visibilities by (uv tile, cell in
 // the tile): LSD radix with digits of up to DMAX bits (two passes up to about
-// 2040^2 cells, three beyond), so a tile's visibilities are grouped by cell
+// 500^2 cells, three beyond), so a tile's visibilities are grouped by cell
 // whatever the input order (baseline-major tracks or time-major snapshots)
 // and keep their input order inside a cell: the gridded sums are reproducible
-// run to run.  A pass is per-chunk digit histograms (digit-major) -> exclusive
-// scan -> order-preserving scatter.
-constexpr int RT = 4096;               // visibilities per sort chunk (256 threads x 16)
-constexpr int DMAX = 11;               // widest digit: 2048 bins
+// run to run.  The input of a pass is cut into two slices an SM; a pass counts
+// the digits of every slice (k_plan_hist), turns the counts into the slices'
+// places in every digit's run (k_plan_offsets) and then moves positions, indices
+// and keys together (k_plan_scatter).
+constexpr int ST_T = 512;              // threads per CTA
+constexpr int ST_W = ST_T / 32;
+constexpr int ST_R = 8;                // visibilities of a thread at a time
+constexpr int RT = ST_T * ST_R;        // a chunk: what a CTA sorts in shared memory at a time
+constexpr int DMAX = 9;                // widest digit: 512 bins
 constexpr int CB = 8;                  // key bits of the cell inside its tile (TS x TS = 2^CB)
 static_assert(TS * TS == 1 << CB, "tile cells must fill CB bits");
+static_assert(1 << DMAX <= ST_T, "one digit a thread");
 
-// Key of position p given its quotients q = (u / dU, v / dU) in binary32, round to nearest.
-__device__ __forceinline__ uint32_t key_from_q(const GridGeom &G, float2 p, float2 q, uint32_t key_none) {
-    if (!(isfinite(p.x) && isfinite(p.y))) return key_none;
-    if (!(fabsf(q.x) < 1.0e7f && fabsf(q.y) < 1.0e7f)) return key_none;
-    const int cx = (int)floorf(__fadd_rn(q.x, 0.5f));
-    const int cy = (int)floorf(__fadd_rn(q.y, 0.5f));
-    const int kx = cx + G.off, ky = cy + G.off;
-    if (kx < 0 || kx >= G.ks || ky < 0 || ky >= G.ks) return key_none;
-    const uint32_t tile = (uint32_t)((ky / TS) * G.tt + kx / TS);
-    return tile << CB | (uint32_t)((ky % TS) * TS + kx % TS);
+// u / dU rounded to nearest: q0 = u y with y = RN(1 / dU), its exact remainder and one correction,
+// q = RN(q0 + RN(u - q0 dU) y), which Markstein's theorem (IBM J. Res. Dev. 34, 1990) makes the
+// correctly rounded quotient unless dU's significand is all ones (by_inv is false then).  Three
+// instructions; where q0 overflows the result is NaN, and no cell either way.
+__device__ __forceinline__ float quotient(const GridGeom &G, float u) {
+    if (!G.by_inv) return __fdiv_rn(u, G.du);
+    const float q0 = __fmul_rn(u, G.inv_du);
+    return __fmaf_rn(__fmaf_rn(-q0, G.du, u), G.inv_du, q0);
 }
 
 __device__ __forceinline__ float2 quotients(const GridGeom &G, float2 p) {
-    return make_float2(__fdiv_rn(p.x, G.du), __fdiv_rn(p.y, G.du));
+    return make_float2(quotient(G, p.x), quotient(G, p.y));
+}
+
+// Key of the position with quotients q = (u / dU, v / dU); key_none for non-finite and far ones.
+__device__ __forceinline__ uint32_t key_from_q(const GridGeom &G, float2 q, uint32_t key_none) {
+    if (!(fabsf(q.x) < 1.0e7f && fabsf(q.y) < 1.0e7f)) return key_none;
+    const uint32_t kx = (uint32_t)((int)floorf(__fadd_rn(q.x, 0.5f)) + G.off);
+    const uint32_t ky = (uint32_t)((int)floorf(__fadd_rn(q.y, 0.5f)) + G.off);
+    if (kx >= (uint32_t)G.ks || ky >= (uint32_t)G.ks) return key_none;
+    const uint32_t tile = (ky / TS) * (uint32_t)G.tt + kx / TS;
+    return tile << CB | (ky % TS) * TS + kx % TS;
 }
 
 __device__ __forceinline__ uint32_t cell_key(const GridGeom &G, float2 p, uint32_t key_none) {
-    return key_from_q(G, p, quotients(G, p), key_none);
-}
-
-// One CTA per chunk: the (tile, cell) key of every visibility (key_none for
-// non-finite or off-grid positions) and the chunk's histogram of the first
-// digit (nbins bins; digit = key & dmask), added once per distinct digit in a
-// warp.  1024 threads, RT / 1024 visibilities each, all loads in flight.
-constexpr int KT = 1024;
-__global__ void __launch_bounds__(KT) k_plan_keys(GridGeom G, int64_t n_vis, const float2 *__restrict__ uv,
-                                                  uint32_t *__restrict__ keys, uint32_t key_none,
-                                                  int nbins, uint32_t dmask, int nchunks,
-                                                  uint32_t *__restrict__ rhist) {
-    __shared__ uint32_t h[1 << DMAX];
-    const int lane = threadIdx.x & 31;
-    for (int d = threadIdx.x; d < nbins; d += KT) h[d] = 0;
-    __syncthreads();
-    const int64_t c0 = (int64_t)blockIdx.x * RT;
-    float2 pv[RT / KT];
-#pragma unroll
-    for (int k = 0; k < RT / KT; ++k) {
-        const int64_t i = c0 + k * KT + threadIdx.x;
-        pv[k] = i < n_vis ? uv[i] : make_float2(0.f, 0.f);
-    }
-#pragma unroll
-    for (int k = 0; k < RT / KT; ++k) {
-        const int64_t i = c0 + k * KT + threadIdx.x;
-        const bool on = i < n_vis;
-        uint32_t key = 0xffffffffu;
-        if (on) {
-            key = cell_key(G, pv[k], key_none);
-            keys[i] = key;
-        }
-        const uint32_t dig = on ? key & dmask : 0x10000000u + lane;
-        const unsigned peers = __match_any_sync(FULL, dig);
-        if (on && lane == __ffs(peers) - 1) atomicAdd(&h[dig], (uint32_t)__popc(peers));
-    }
-    __syncthreads();
-    for (int d = threadIdx.x; d < nbins; d += KT) rhist[(int64_t)d * nchunks + blockIdx.x] = h[d];
+    return key_from_q(G, quotients(G, p), key_none);
 }
 
 // Block-wide exclusive scan of one value per thread (blockDim.x a multiple of 32, at most 1024).
@@ -177,224 +161,221 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t *s
     return warp_base + x - v;
 }
 
-// Order-preserving scatter of one chunk (RT items, ST_W warps; warp w owns
-// the contiguous [w RT/ST_W, (w+1) RT/ST_W) of the chunk).  One sweep ranks
-// every item among the warp's earlier items of its digit (__match_any_sync,
-// lower lanes first) and counts the warp's digits; a prefix over (digit,
-// warp) then gives every item its place in the chunk ordered by digit, where
-// it is staged in shared memory, and the staged chunk is written out in that
-// order: each digit's run goes to consecutive addresses, starting where the
-// scanned histogram puts this chunk's part of the digit (local scan + its
-// block's offset).  vin == nullptr means the identity (first pass); on the
-// last pass (uv_out != nullptr) the sorted original indices and positions
-// are written instead of keys.  Before the last pass, the next pass's
-// per-chunk digit histogram (digit at shift + dw of every placed key, chunk
-// = position / RT) is counted into nhist, which must hold zeros: one global
-// add per distinct (digit, chunk) in a warp.
-constexpr int ST_W = 16;                 // warps per scatter CTA
-constexpr int ST_T = ST_W * 32;
-constexpr int ST_R = RT / ST_T;          // items per thread
-constexpr int ST_D = (1 << DMAX) / ST_T; // digits per thread at most
-__host__ __device__ constexpr int scatter_row(int nbins) { return (nbins + 7) & ~7; }
-__host__ __device__ constexpr size_t scatter_smem(int nbins) {
-    return sizeof(uint32_t) * (2 * RT + 2 * (size_t)scatter_row(nbins)) +
-           sizeof(uint16_t) * ST_W * (size_t)scatter_row(nbins);
+// hist[digit][slice]: the digit counts of one slice (shared-memory counters, whose hardware adds
+// merge equal digits of a warp), from the positions (first pass) or the keys.
+template <bool FIRST>
+__global__ void __launch_bounds__(ST_T) k_plan_hist(GridGeom G, int64_t n, int64_t per_slice,
+                                                    const float2 *__restrict__ uv, const uint32_t *__restrict__ keys,
+                                                    uint32_t key_none, int shift, int dw, uint32_t *__restrict__ hist) {
+    __shared__ uint32_t h[1 << DMAX];
+    const int nb = 1 << dw;
+    if ((int)threadIdx.x < nb) h[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t b0 = blockIdx.x * per_slice;
+    const int cnt = (int)(min(n, b0 + per_slice) - b0);   // a slice is far below 2^31
+    constexpr int K = 4;                 // visibilities of a thread in flight
+    for (int b = threadIdx.x; b < cnt; b += ST_T * K) {
+        uint32_t key[K];
+        if (FIRST) {
+            float2 p[K];
+#pragma unroll
+            for (int k = 0; k < K; ++k) p[k] = b + k * ST_T < cnt ? uv[b0 + b + k * ST_T] : make_float2(0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < K; ++k) key[k] = cell_key(G, p[k], key_none);
+        } else {
+#pragma unroll
+            for (int k = 0; k < K; ++k) key[k] = b + k * ST_T < cnt ? keys[b0 + b + k * ST_T] : 0u;
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            if (b + k * ST_T < cnt) atomicAdd(&h[(key[k] >> shift) & (uint32_t)(nb - 1)], 1u);
+    }
+    __syncthreads();
+    if ((int)threadIdx.x < nb) hist[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = h[threadIdx.x];
 }
-__global__ void __launch_bounds__(ST_T, 2) k_radix_scatter(const uint32_t *__restrict__ kin,
-                                                        const uint32_t *__restrict__ vin, int64_t n,
-                                                        int shift, int nbins, uint32_t dmask, int nchunks,
-                                                        const uint32_t *__restrict__ offs,
-                                                        const uint32_t *__restrict__ bsum,
-                                                        uint32_t *__restrict__ kout,
-                                                        uint32_t *__restrict__ vout,
-                                                        const float2 *__restrict__ uv,
-                                                        float2 *__restrict__ uv_out, int dw,
-                                                        uint32_t *__restrict__ nhist) {
+
+// One warp per digit: the counts of its slices become their exclusive sums, in place, and total[digit].
+__global__ void __launch_bounds__(256) k_plan_offsets(int nb, int slices, uint32_t *__restrict__ hist,
+                                                      uint32_t *__restrict__ total) {
+    const int d = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (d >= nb) return;
+    uint32_t *h = hist + (size_t)d * slices;
+    uint32_t carry = 0;
+    for (int c0 = 0; c0 < slices; c0 += 32 * 4) {
+        uint32_t v[4], s = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int c = c0 + 4 * lane + k;
+            v[k] = c < slices ? h[c] : 0u;
+            s += v[k];
+        }
+        uint32_t x = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(FULL, x, o);
+            if (lane >= o) x += y;
+        }
+        uint32_t run = carry + x - s;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int c = c0 + 4 * lane + k;
+            if (c < slices) h[c] = run;
+            run += v[k];
+        }
+        carry += __shfl_sync(FULL, x, 31);
+    }
+    if (lane == 0) total[d] = carry;
+}
+
+// One slice of a pass, stably by its digit, a chunk of up to RT visibilities at a time (warp w
+// owns a contiguous part of the chunk):
+//  - every item's rank among its warp's earlier items of its digit, on top of the warp's running
+//    count of the digit: the lanes of one digit by __match_any_sync for every other row and by a
+//    ballot per digit bit for the rest, which spreads the work over the two units that do them (all
+//    matches: 77 cycles a row and SM, all ballots: 1 % slower overall than half and half).  DW is a
+//    template parameter: with a runtime width the tests between the ballots doubled the kernel's
+//    instructions;
+//  - the chunk staged in shared memory in digit order and written out in that order: consecutive
+//    threads, consecutive addresses within a run.
+// FIRST: keys are computed from the positions and the indices are the identity; LAST: no keys are
+// written.  Positions travel with the indices, so no pass gathers, and no CTA waits for another (a
+// single sweep with look-back spent 8 of 20 us a pass waiting at 1e6 visibilities).  Bound by
+// instruction issue and the latency of a chunk's phases.
+__host__ __device__ constexpr size_t sort_smem(int nb) {
+    return (sizeof(float2) + 2 * sizeof(uint32_t)) * RT + 2 * sizeof(uint32_t) * nb + sizeof(uint16_t) * ST_W * nb;
+}
+template <int DW, bool FIRST, bool LAST>
+__global__ void __launch_bounds__(ST_T, 2) k_plan_scatter(GridGeom G, int64_t n, int64_t per_slice,
+                                                          const float2 *__restrict__ uv_in,
+                                                          const uint32_t *__restrict__ idx_in,
+                                                          const uint32_t *__restrict__ key_in, uint32_t key_none, int shift,
+                                                          const uint32_t *__restrict__ offs,
+                                                          const uint32_t *__restrict__ total, float2 *__restrict__ uv_out,
+                                                          uint32_t *__restrict__ idx_out, uint32_t *__restrict__ key_out) {
     extern __shared__ __align__(16) uint8_t ssm[];
-    const int row = scatter_row(nbins);                  // nbins rounded up to 8 (16-byte rows)
-    uint32_t *skey = (uint32_t *)ssm;                    // [RT] the chunk ordered by digit
-    uint32_t *sval = skey + RT;                          // [RT]
-    uint32_t *gbase = sval + RT;                         // [row] global position of local 0 for the digit
-    uint32_t *lstart = gbase + row;                      // [row] the digit's first local position
-    uint16_t *wcnt = (uint16_t *)(lstart + row);         // [ST_W][row] per-warp counts, then offsets
+    constexpr int nb = 1 << DW;
+    float2 *suv = (float2 *)ssm;                         // [RT] the chunk ordered by digit
+    uint32_t *sidx = (uint32_t *)(suv + RT);             // [RT]
+    uint32_t *skey = sidx + RT;                          // [RT]
+    uint32_t *gbase = skey + RT;                         // [nb] global position of local 0 for the digit
+    uint32_t *lstart = gbase + nb;                       // [nb] the digit's first local position
+    uint16_t *wcnt = (uint16_t *)(lstart + nb);          // [ST_W][nb] per-warp counts, then offsets
     __shared__ uint32_t sh[32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tid = threadIdx.x;
     const unsigned lt = (1u << lane) - 1u;
-    const int64_t c0 = (int64_t)blockIdx.x * RT;
-    const int64_t w0 = c0 + warp * (RT / ST_W);
-    const int nloc = (int)min((int64_t)RT, n - c0);
-    // every load in flight at once: keys, values, this thread's digit offsets
-    uint32_t kv[ST_R], vv[ST_R];
-#pragma unroll
-    for (int k = 0; k < ST_R; ++k) {
-        const int64_t e = w0 + k * 32 + lane;
-        kv[k] = e < n ? kin[e] : 0u;
-        vv[k] = vin ? (e < n ? vin[e] : 0u) : (uint32_t)e;
+    const int64_t b0 = blockIdx.x * per_slice;
+    const int size = (int)(min(n, b0 + per_slice) - b0);
+    uv_in += b0;
+    if (!FIRST) {
+        idx_in += b0;
+        key_in += b0;
     }
-    const int d0 = threadIdx.x * ST_D;   // this thread's digits [d0, d0 + ST_D)
+    // thread d < nb: global position of the digit's next item
+    uint32_t tot, next = block_exclusive_scan(tid < nb ? total[tid] : 0u, sh, tot);
+    if (tid < nb) next += offs[(size_t)tid * gridDim.x + blockIdx.x];
+    uint16_t *mycnt = wcnt + warp * nb;
+    for (int c0 = 0; c0 < size; c0 += RT) {
+        const int nloc = min(RT, size - c0);
+        const int rows = (nloc + ST_T - 1) / ST_T;       // 32-item rows of a warp
+        const int w0 = warp * rows * 32;
+        float2 p[ST_R];
+        uint32_t ix[ST_R], key[ST_R], rk[ST_R / 2];      // rk: two ranks
 #pragma unroll
-    for (int j = 0; j < ST_D; ++j) {
-        const int64_t e = (int64_t)(d0 + j) * nchunks + blockIdx.x;
-        if (d0 + j < nbins) gbase[d0 + j] = offs[e] + bsum[e / 4096];
-    }
-    for (int i = threadIdx.x; i < ST_W * row / 8; i += ST_T) ((uint4 *)wcnt)[i] = make_uint4(0u, 0u, 0u, 0u);
-    __syncthreads();
-    // rank of every item among its warp's earlier items of the same digit
-    // (below 256: two 16-bit ranks to a register)
-    uint32_t rk[ST_R / 2];
+        for (int k = 0; k < ST_R; ++k) {
+            const int e = w0 + k * 32 + lane;
+            const bool on = k < rows && e < nloc;
+            p[k] = on ? uv_in[c0 + e] : make_float2(0.f, 0.f);
+            ix[k] = FIRST ? (uint32_t)b0 + (uint32_t)(c0 + e) : on ? idx_in[c0 + e] : 0u;
+            if (!FIRST) key[k] = on ? key_in[c0 + e] : 0u;
+        }
+        __syncthreads();   // the chunk before has been written out
+        for (int i = tid; i < ST_W * nb / 8; i += ST_T) ((uint4 *)wcnt)[i] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
 #pragma unroll
-    for (int k = 0; k < ST_R; ++k) {
-        const bool on = w0 + k * 32 + lane < n;
-        const uint32_t d = on ? (kv[k] >> shift) & dmask : 0x10000u + lane;
-        const unsigned peers = __match_any_sync(FULL, d);
-        uint32_t before = 0;
-        if (on) before = wcnt[warp * row + d];
-        const uint32_t rank = before + (uint32_t)__popc(peers & lt);
-        if (k % 2 == 0) rk[k / 2] = rank;
-        else rk[k / 2] |= rank << 16;
-        __syncwarp();
-        if (on && lane == __ffs(peers) - 1) wcnt[warp * row + d] = (uint16_t)(before + __popc(peers));
-        __syncwarp();
-    }
-    __syncthreads();
-    // per digit: offsets of the warps inside its run; the runs' local starts
-    uint32_t cnt[ST_D], mine = 0;
+        for (int k = 0; k < ST_R; ++k)
+            if (k < rows) {
+                const bool on = w0 + k * 32 + lane < nloc;
+                if (FIRST) key[k] = cell_key(G, p[k], key_none);
+                const uint32_t d = (key[k] >> shift) & (uint32_t)(nb - 1);
+                unsigned peers;
+                if (k % 2) {
+                    peers = __match_any_sync(FULL, on ? d : 1u << DW);
+                } else {
+                    peers = __ballot_sync(FULL, on);
 #pragma unroll
-    for (int j = 0; j < ST_D; ++j) {
-        const int d = d0 + j;
-        uint32_t run = 0;
-        if (d < nbins) {
+                    for (int b = 0; b < DW; ++b) {
+                        const bool bit = (d >> b) & 1u;
+                        const unsigned v = __ballot_sync(FULL, bit);
+                        peers &= bit ? v : ~v;
+                    }
+                }
+                const uint32_t before = mycnt[d], rank = before + (uint32_t)__popc(peers & lt);
+                if (k % 2 == 0) rk[k / 2] = rank;
+                else rk[k / 2] |= rank << 16;
+                __syncwarp();
+                if (on && lane == __ffs(peers) - 1) mycnt[d] = (uint16_t)(before + __popc(peers));
+                __syncwarp();
+            }
+        __syncthreads();
+        // per digit: offsets of the warps inside its run; the run's local start and global place
+        uint32_t cnt = 0;
+        if (tid < nb) {
+            uint32_t c[ST_W];
+#pragma unroll
+            for (int w = 0; w < ST_W; ++w) c[w] = wcnt[w * nb + tid];
 #pragma unroll
             for (int w = 0; w < ST_W; ++w) {
-                const uint32_t c = wcnt[w * row + d];
-                wcnt[w * row + d] = (uint16_t)run;
-                run += c;
+                wcnt[w * nb + tid] = (uint16_t)cnt;
+                cnt += c[w];
             }
         }
-        cnt[j] = run;
-        mine += run;
-    }
-    uint32_t total;
-    uint32_t ls = block_exclusive_scan(mine, sh, total);
-#pragma unroll
-    for (int j = 0; j < ST_D; ++j) {
-        const int d = d0 + j;
-        if (d < nbins) {
-            lstart[d] = ls;
-            gbase[d] -= ls;   // global position = gbase[d] + local position
+        const uint32_t ls = block_exclusive_scan(cnt, sh, tot);
+        if (tid < nb) {
+            lstart[tid] = ls;
+            gbase[tid] = next - ls;
+            next += cnt;
         }
-        ls += cnt[j];
-    }
-    __syncthreads();
+        __syncthreads();
 #pragma unroll
-    for (int k = 0; k < ST_R; ++k) {
-        if (w0 + k * 32 + lane < n) {
-            const uint32_t d = (kv[k] >> shift) & dmask;
-            const uint32_t L = lstart[d] + wcnt[warp * row + d] + ((rk[k / 2] >> (16 * (k % 2))) & 0xffffu);
-            skey[L] = kv[k];
-            sval[L] = vv[k];
-        }
-    }
-    __syncthreads();
-    // write-out in digit order: consecutive threads, consecutive addresses within a run
-    if (uv_out) {
-        float2 pv[ST_R];
-        uint32_t gp[ST_R], vl[ST_R];
+        for (int k = 0; k < ST_R; ++k)
+            if (k < rows && w0 + k * 32 + lane < nloc) {
+                const uint32_t d = (key[k] >> shift) & (uint32_t)(nb - 1);
+                const uint32_t L = lstart[d] + mycnt[d] + ((rk[k / 2] >> (16 * (k % 2))) & 0xffffu);
+                suv[L] = p[k];
+                sidx[L] = ix[k];
+                skey[L] = key[k];
+            }
+        __syncthreads();
 #pragma unroll
         for (int k = 0; k < ST_R; ++k) {
-            const int L = k * ST_T + threadIdx.x;
+            const int L = k * ST_T + tid;
             if (L < nloc) {
-                const uint32_t key = skey[L];
-                vl[k] = sval[L];
-                gp[k] = gbase[(key >> shift) & dmask] + (uint32_t)L;
-                pv[k] = uv[vl[k]];
+                const uint32_t kk = skey[L], pos = gbase[(kk >> shift) & (uint32_t)(nb - 1)] + (uint32_t)L;
+                uv_out[pos] = suv[L];
+                idx_out[pos] = sidx[L];
+                if (!LAST) key_out[pos] = kk;
             }
-        }
-#pragma unroll
-        for (int k = 0; k < ST_R; ++k) {
-            if (k * ST_T + (int)threadIdx.x < nloc) {
-                vout[gp[k]] = vl[k];
-                uv_out[gp[k]] = pv[k];
-            }
-        }
-        return;
-    }
-#pragma unroll
-    for (int k = 0; k < ST_R; ++k) {
-        const int L = k * ST_T + threadIdx.x;
-        const bool on = L < nloc;
-        uint32_t key = 0, pos = 0;
-        if (on) {
-            key = skey[L];
-            pos = gbase[(key >> shift) & dmask] + (uint32_t)L;
-            kout[pos] = key;
-            vout[pos] = sval[L];
-        }
-        if (nhist) {   // (next digit, destination chunk): below 2^11 x 2^20 for valid lanes
-            const uint32_t d2 = (key >> (shift + dw)) & (uint32_t)((1 << dw) - 1);
-            const uint32_t h2 = on ? d2 << 20 | pos / RT : 0x80000000u + lane;
-            const unsigned p2 = __match_any_sync(FULL, h2);
-            if (on && lane == __ffs(p2) - 1)
-                atomicAdd(&nhist[(int64_t)d2 * nchunks + pos / RT], (uint32_t)__popc(p2));
         }
     }
 }
 
-// Exclusive scan of len values, 4096 per 1024-thread block: every block scans
-// its part into out and writes its total; the last block to finish (ticket)
-// scans the totals in place into block offsets (so element e's exclusive
-// prefix is out[e] + bsum[e / 4096]) and re-arms the ticket.  zero_in, when
-// given, is the input array itself, cleared once read (the next radix pass
-// counts into it).
-__global__ void __launch_bounds__(1024) k_scan(const uint32_t *in, int64_t len,
-                                               uint32_t *__restrict__ out, uint32_t *__restrict__ bsum,
-                                               unsigned *__restrict__ ticket, uint32_t *zero_in) {
-    __shared__ uint32_t sh[32];
-    __shared__ bool last;
-    const int64_t base = (int64_t)blockIdx.x * 4096 + threadIdx.x * 4;
-    uint32_t v[4];
-    uint32_t s = 0;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        v[k] = base + k < len ? in[base + k] : 0u;
-        s += v[k];
+using ScatterFn = void (*)(GridGeom, int64_t, int64_t, const float2 *, const uint32_t *, const uint32_t *, uint32_t, int,
+                           const uint32_t *, const uint32_t *, float2 *, uint32_t *, uint32_t *);
+template <int DW>
+ScatterFn scatter_of(bool first, bool last) {
+    if constexpr (DW == DMAX) {   // a single pass: 9 key bits
+        if (first && last) return k_plan_scatter<DW, true, true>;
     }
-    if (zero_in) {   // the same array as in
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (base + k < len) zero_in[base + k] = 0u;
-    }
-    uint32_t total;
-    uint32_t pre = block_exclusive_scan(s, sh, total);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        if (base + k < len) out[base + k] = pre;
-        pre += v[k];
-    }
-    if (threadIdx.x == 0) {
-        bsum[blockIdx.x] = total;
-        __threadfence();
-        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    uint32_t carry = 0;
-    for (int64_t b = 0; b < gridDim.x; b += 1024) {
-        const int64_t i = b + threadIdx.x;
-        const uint32_t x = i < gridDim.x ? __ldcg(bsum + i) : 0u;
-        uint32_t t;
-        const uint32_t p = block_exclusive_scan(x, sh, t);
-        if (i < gridDim.x) bsum[i] = carry + p;
-        carry += t;
-    }
-    if (threadIdx.x == 0) *ticket = 0u;
+    return first ? k_plan_scatter<DW, true, false> : last ? k_plan_scatter<DW, false, true> : k_plan_scatter<DW, false, false>;
 }
-
-__global__ void k_scan_add(uint32_t *__restrict__ out, int64_t len,
-                           const uint32_t *__restrict__ block_sums) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < len) out[i] += block_sums[i / 4096];
+ScatterFn scatter_of(int dw, bool first, bool last) {
+    switch (dw) {   // at least 9 key bits, so at least 5 of a digit
+        case 5: return scatter_of<5>(first, last);
+        case 6: return scatter_of<6>(first, last);
+        case 7: return scatter_of<7>(first, last);
+        case 8: return scatter_of<8>(first, last);
+        default: return scatter_of<9>(first, last);
+    }
 }
 
 // ------------------------------------------------------------------ accumulation
@@ -404,15 +385,16 @@ __global__ void k_scan_add(uint32_t *__restrict__ out, int64_t len,
 // once and staged in shared memory, and the unit is cut into tasks: runs of
 // one cell, also cut at every CHUNK-th item of the unit, so a task holds at
 // most CHUNK visibilities.  A warp takes a task; lane (dy, q) owns the
-// footprint cells (2q, dy) and (2q+1, dy) of the (2r+1)^2 around the run's
-// cell and sums w = wx wy, w Re V, w Im V over the run with packed FP32x2
+// footprint cells (q, dy) and (q + 4, dy) of the (2r+1)^2 around the run's
+// cell (its lanes' FP64 adds cover whole sectors of a grid row) and sums w = wx wy, w Re V, w Im V over the run with packed FP32x2
 // arithmetic (plain blocks of GFOLD, as two interleaved chains, folded into
 // Kahan sums; a fixed order), then adds its cells to the FP64 grid.  No
 // shared accumulators: runs never wait on one another, whether the cell is
 // dense (long runs) or sparse.
 //
-// Staged record of a visibility (RS floats): wx[0..7] (zero beyond 2r),
-// (wy[d], wy[d]) for d = 0..6, two pad floats, (Re V, Re V, Im V, Im V).
+// Staged record of a visibility (RS floats): wx of columns 0, 4, 1, 5, 2, 6, 3
+// (a lane's two columns are adjacent; zero beyond 2r), a zero, (wy[d], wy[d])
+// for d = 0..6, two pad floats, (Re V, Re V, Im V, Im V).
 constexpr int GT = 256;          // threads per gridding CTA (8 warps x UMAX/8 items)
 // What the third (and fourth) accumulator plane of a cell holds: the weight sum
 // (GW_SUM), the number N_g of visibilities entered (GW_COUNT, Eq. vg), or the
@@ -428,16 +410,18 @@ constexpr size_t GRID_SMEM = UMAX * sizeof(float) * RS + sizeof(uint32_t) * UMAX
 
 // The double with the value of x, built with integer operations only (GB300's
 // FP64 pipe is narrow: one hardware conversion per flushed value is what kept
-// it busy).  Exact for normal, infinite and NaN x; subnormal x (|x| < 2^-126)
-// become a zero of the same sign.
+// it busy).  widen: normal x.  is_special: x is zero, subnormal, infinite or NaN, which widen_any
+// takes too (subnormal x, |x| < 2^-126, become a zero of the same sign).
 __device__ __forceinline__ double widen(float x) {
     const uint32_t b = __float_as_uint(x);
-    const uint32_t e = (b >> 23) & 255u;
-    const uint32_t sign = b & 0x80000000u;
+    return __hiloint2double((int)((((int)b >> 3) & 0x8fffffff) + 0x38000000), (int)(b << 29));
+}
+__device__ __forceinline__ bool is_special(float x) { return ((__float_as_uint(x) + 0x00800000u) & 0x7f000000u) == 0u; }
+__device__ __noinline__ double widen_any(float x) {
+    const uint32_t b = __float_as_uint(x), e = (b >> 23) & 255u, sign = b & 0x80000000u;
     const uint32_t eh = e == 255u ? 2047u : e + (1023u - 127u);
     const uint32_t hi = e == 0u ? sign : sign | (eh << 20) | ((b >> 3) & 0xFFFFFu);
-    const uint32_t lo = e == 0u ? 0u : b << 29;
-    return __hiloint2double((int)hi, (int)lo);
+    return __hiloint2double((int)hi, (int)(e == 0u ? 0u : b << 29));
 }
 
 __device__ __forceinline__ void kahan_add2(float2 &s, float2 &c, float2 x) {
@@ -487,6 +471,25 @@ __device__ __forceinline__ void load_unit(UnitIn &in, int64_t u, int64_t nu, int
     }
 }
 
+// A run's sums of one footprint cell into the FP64 grid.
+template <int WM>
+__device__ __forceinline__ void grid_add(double *__restrict__ re, double *__restrict__ im, double *__restrict__ w,
+                                         double *__restrict__ w2, float vre, float vim, float vw, float vw2, double run) {
+    const bool odd = is_special(vre) || is_special(vim) || (WM != GW_COUNT && is_special(vw)) ||
+                     (WM == GW_SUM_SQ && is_special(vw2));
+    if (!odd) {
+        atomicAdd(re, widen(vre));
+        atomicAdd(im, widen(vim));
+        atomicAdd(w, WM == GW_COUNT ? run : widen(vw));
+        if (WM == GW_SUM_SQ) atomicAdd(w2, widen(vw2));
+    } else {
+        atomicAdd(re, widen_any(vre));
+        atomicAdd(im, widen_any(vim));
+        atomicAdd(w, WM == GW_COUNT ? run : widen_any(vw));
+        if (WM == GW_SUM_SQ) atomicAdd(w2, widen_any(vw2));
+    }
+}
+
 template <int WM>
 __global__ void __launch_bounds__(GT, 3) k_grid(GridGeom G, int64_t n_vis, uint32_t key_none,
                                              const float2 *__restrict__ s_uv,
@@ -501,12 +504,13 @@ __global__ void __launch_bounds__(GT, 3) k_grid(GridGeom G, int64_t n_vis, uint3
     uint32_t *skey = (uint32_t *)(st + UMAX * RS);                     // [UMAX] key of every item
     uint16_t *tstart = (uint16_t *)(skey + UMAX);                      // [UMAX + 1] first item of each task
     __shared__ uint32_t wsum_s[8], wvalid_s[8];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = GT / 32;
+    __shared__ int next_s;   // next task of the unit
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int r = G.r, fw = 2 * r + 1;
     const bool gauss = G.kernel == ABS_KERNEL_GAUSS;
-    // this lane's footprint cells: (2q, dy) and (2q + 1, dy)
-    const int dy = lane >> 2, q2 = 2 * (lane & 3);
-    const bool on_a = lane < 28 && dy < fw && q2 < fw, on_b = on_a && q2 + 1 < fw;
+    // this lane's footprint cells: (qx, dy) and (qx + 4, dy)
+    const int dy = lane >> 2, qx = lane & 3;
+    const bool on_a = dy < fw && qx < fw, on_b = on_a && qx + 4 < fw;
     const int64_t nu = cdiv(n_vis, UMAX);
     UnitIn nxt;
     load_unit(nxt, blockIdx.x, nu, n_vis, s_uv, s_idx, warp, lane);
@@ -529,7 +533,7 @@ __global__ void __launch_bounds__(GT, 3) k_grid(GridGeom G, int64_t n_vis, uint3
             valid[h] = false;
             if (t < total) {
                 q[h] = quotients(G, cur.p[h]);
-                const uint32_t key = key_from_q(G, cur.p[h], q[h], key_none);
+                const uint32_t key = key_from_q(G, q[h], key_none);
                 skey[t] = key;
                 valid[h] = key != key_none;
             }
@@ -559,7 +563,10 @@ __global__ void __launch_bounds__(GT, 3) k_grid(GridGeom G, int64_t n_vis, uint3
         const unsigned lt = (1u << lane) - 1u;
         if (ts[0]) tstart[wbase + __popc(b0 & lt)] = (uint16_t)(warp * 64 + lane);
         if (ts[1]) tstart[wbase + __popc(b0) + __popc(b1 & lt)] = (uint16_t)(warp * 64 + 32 + lane);
-        if (threadIdx.x == 0) tstart[ntask] = (uint16_t)nvalid;
+        if (threadIdx.x == 0) {
+            tstart[ntask] = (uint16_t)nvalid;
+            next_s = GT / 32;   // the warps' first tasks are their own numbers
+        }
         // staging: weights and visibility of every valid item, in place
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -572,24 +579,21 @@ __global__ void __launch_bounds__(GT, 3) k_grid(GridGeom G, int64_t n_vis, uint3
                 // relative size 2^-24, so one rounding of its own does not matter
                 const float fxl = __fmul_rn(fmaf(-qq.x, G.du, p.x), G.inv_du);
                 const float fyl = __fmul_rn(fmaf(-qq.y, G.du, p.y), G.inv_du);
-                float *rec = st + t * RS;
-                float wx[8], wy[8];
+                const float2 nf = make_float2(-fxh, -fyh), nfl = make_float2(-fxl, -fyl);
+                float2 w[7];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    wx[k] = wy[k] = 0.f;
-                    if (k < fw) {
-                        const float d = (float)(k - r);
-                        wx[k] = gauss ? wexp(d, fxh, fxl, G.s_hi, G.s_lo) : 1.f;
-                        wy[k] = gauss ? wexp(d, fyh, fyl, G.s_hi, G.s_lo) : 1.f;
-                    }
+                for (int k = 0; k < 7; ++k) {
+                    w[k] = make_float2(0.f, 0.f);
+                    if (k < fw) w[k] = gauss ? wexp2((float)(k - r), nf, nfl, G.s_hi, G.s_lo) : make_float2(1.f, 1.f);
                 }
-                ((float4 *)rec)[0] = make_float4(wx[0], wx[1], wx[2], wx[3]);
-                ((float4 *)rec)[1] = make_float4(wx[4], wx[5], wx[6], wx[7]);
+                float4 *rec = (float4 *)(st + t * RS);
+                rec[0] = make_float4(w[0].x, w[4].x, w[1].x, w[5].x);
+                rec[1] = make_float4(w[2].x, w[6].x, w[3].x, 0.f);
 #pragma unroll
                 for (int k = 0; k < 3; ++k)
-                    ((float4 *)(rec + R_WY))[k] = make_float4(wy[2 * k], wy[2 * k], wy[2 * k + 1], wy[2 * k + 1]);
-                ((float2 *)(rec + R_WY))[6] = make_float2(wy[6], wy[6]);
-                ((float4 *)(rec + R_V))[0] = make_float4(v[h].x, v[h].x, v[h].y, v[h].y);
+                    rec[R_WY / 4 + k] = make_float4(w[2 * k].y, w[2 * k].y, w[2 * k + 1].y, w[2 * k + 1].y);
+                ((float2 *)(rec + R_WY / 4 + 3))[0] = make_float2(w[6].y, w[6].y);
+                rec[R_V / 4] = make_float4(v[h].x, v[h].x, v[h].y, v[h].y);
             }
         }
         // the next unit's visibilities: its indices have arrived by now
@@ -597,12 +601,14 @@ __global__ void __launch_bounds__(GT, 3) k_grid(GridGeom G, int64_t n_vis, uint3
         for (int h = 0; h < 2; ++h)
             if (u + gridDim.x < nu && warp * 64 + h * 32 + lane < nxt.cnt) vn[h] = vis[nxt.idx[h]];
         __syncthreads();
-        if (on_a) {   // lanes without a footprint cell take no part in the sums
-            for (int tk = warp; tk < (int)ntask; tk += nwarps) {
+        for (int tk = warp, nx = 0; tk < (int)ntask; tk = nx) {
+            if (lane == 0) nx = atomicAdd(&next_s, 1);   // tasks differ in length: the next free one
+            nx = __shfl_sync(FULL, nx, 0);
+            if (on_a) {   // lanes without a footprint cell take no part in the sums
                 const int j_begin = tstart[tk], j_end = tstart[tk + 1];
                 const float2 z = make_float2(0.f, 0.f);
                 float2 sre = z, cre = z, sim = z, cim = z, sw = z, cw = z, sw2 = z, cw2 = z;
-                const float *lw = st + q2, *lwy = st + R_WY + 2 * dy, *lv = st + R_V;
+                const float *lw = st + 2 * qx, *lwy = st + R_WY + 2 * dy, *lv = st + R_V;
                 for (int j0 = j_begin; j0 < j_end; j0 += GFOLD) {   // plain blocks of GFOLD, folded into Kahan sums
                     float2 bre = z, bim = z, bw = z, bw2 = z;
                     if (j0 + GFOLD <= j_end) {
@@ -629,109 +635,72 @@ __global__ void __launch_bounds__(GT, 3) k_grid(GridGeom G, int64_t n_vis, uint3
                 const uint32_t key = skey[j_begin];
                 const int tile = (int)(key >> CB), loc = (int)(key & (uint32_t)(TS * TS - 1));
                 const int kx = (tile % G.tt) * TS + (loc & (TS - 1)), ky = (tile / G.tt) * TS + (loc >> 4);
-                const int gy = ky - G.off + dy - r;
-                const int gxa = kx - G.off + q2 - r;
-                if (gy < -G.half || gy > G.half) continue;
+                const int gy = ky - G.off + dy - r, gx = kx - G.off + qx - r;
+                if (abs(gy) > G.half) continue;
                 // the run's sums s - c, rounded once to FP32 (relative 2^-24 of the run)
                 const float2 m1 = make_float2(-1.f, -1.f);
                 const float2 vre = __ffma2_rn(cre, m1, sre), vim = __ffma2_rn(cim, m1, sim);
                 const float2 vw = __ffma2_rn(cw, m1, sw), vw2 = __ffma2_rn(cw2, m1, sw2);
-                const double run = (double)(j_end - j_begin);   // visibilities the run enters at the cell
-                if (gxa >= -G.half && gxa <= G.half) {
-                    const int64_t pidx = cell_index(G.n, gxa, gy);
-                    atomicAdd(&acc_re[pidx], widen(vre.x));
-                    atomicAdd(&acc_im[pidx], widen(vim.x));
-                    atomicAdd(&acc_w[pidx], WM == GW_COUNT ? run : widen(vw.x));
-                    if (WM == GW_SUM_SQ) atomicAdd(&acc_w2[pidx], widen(vw2.x));
+                const double run = WM == GW_COUNT ? (double)(j_end - j_begin) : 0.0;   // visibilities entered at the cell
+                const int row = (gy < 0 ? gy + G.n : gy) * G.n;   // n <= 8192: cells fit 32 bits
+                if (abs(gx) <= G.half) {
+                    const int o = row + (gx < 0 ? gx + G.n : gx);
+                    grid_add<WM>(acc_re + o, acc_im + o, acc_w + o, acc_w2 + o, vre.x, vim.x, vw.x, vw2.x, run);
                 }
-                if (on_b && gxa + 1 >= -G.half && gxa + 1 <= G.half) {
-                    const int64_t pidx = cell_index(G.n, gxa + 1, gy);
-                    atomicAdd(&acc_re[pidx], widen(vre.y));
-                    atomicAdd(&acc_im[pidx], widen(vim.y));
-                    atomicAdd(&acc_w[pidx], WM == GW_COUNT ? run : widen(vw.y));
-                    if (WM == GW_SUM_SQ) atomicAdd(&acc_w2[pidx], widen(vw2.y));
+                if (on_b && abs(gx + 4) <= G.half) {
+                    const int o = row + (gx + 4 < 0 ? gx + 4 + G.n : gx + 4);
+                    grid_add<WM>(acc_re + o, acc_im + o, acc_w + o, acc_w2 + o, vre.y, vim.y, vw.y, vw2.y, run);
                 }
             }
         }
     }
 }
 
-// Hermitian mirror and FP32 outputs: G(g) + conj G(-g), W(g) + W(-g).
-__global__ void k_grid_finalize(int n, const double *__restrict__ acc_re,
-                                const double *__restrict__ acc_im,
-                                const double *__restrict__ acc_w,
-                                float2 *__restrict__ grid, float *__restrict__ wsum,
-                                uint8_t *__restrict__ mask) {
-    const int64_t cells = (int64_t)n * n;
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < cells;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        const int ix = (int)(p % n), iy = (int)(p / n);
-        if (ix == n / 2 || iy == n / 2) {
-            grid[p] = make_float2(0.f, 0.f);
-            wsum[p] = 0.f;
-            mask[p] = 0;
-            continue;
-        }
-        const int mx = ix == 0 ? 0 : n - ix, my = iy == 0 ? 0 : n - iy;
-        const int64_t pm = (int64_t)my * n + mx;
-        grid[p] = make_float2((float)(acc_re[p] + acc_re[pm]), (float)(acc_im[p] - acc_im[pm]));
-        wsum[p] = (float)(acc_w[p] + acc_w[pm]);
-        mask[p] = (acc_w[p] > 0.0 || acc_w[pm] > 0.0) ? 1 : 0;   // a filled cell has weight > 0
+// Hermitian mirror and FP32 outputs: G(g) + conj G(-g), W(g) + W(-g).  One thread per cell of the
+// rows 0 .. n/2 (blockIdx.y), which also writes the mirrored cell, so the accumulators are read once.
+// Bound by memory: 24 bytes read and 13 written a cell.
+__global__ void __launch_bounds__(256) k_grid_finalize(int n, const double *__restrict__ acc_re,
+                                                       const double *__restrict__ acc_im,
+                                                       const double *__restrict__ acc_w, float2 *__restrict__ grid,
+                                                       float *__restrict__ wsum, uint8_t *__restrict__ mask) {
+    const int ix = blockIdx.x * 256 + threadIdx.x, iy = blockIdx.y;
+    if (ix >= n) return;
+    const int mx = ix == 0 ? 0 : n - ix, my = iy == 0 ? 0 : n - iy;
+    const int64_t p = (int64_t)iy * n + ix, pm = (int64_t)my * n + mx;
+    float2 g = make_float2(0.f, 0.f);
+    float w = 0.f;
+    uint8_t on = 0;
+    if (ix != n / 2 && iy != n / 2) {
+        const double wa = acc_w[p], wb = acc_w[pm];
+        g = make_float2((float)(acc_re[p] + acc_re[pm]), (float)(acc_im[p] - acc_im[pm]));
+        w = (float)(wa + wb);
+        on = wa > 0.0 || wb > 0.0;   // a filled cell has weight > 0
     }
-}
-
-
-// Filled mask only, for the estimate path (which transforms straight from the
-// FP64 accumulators): a cell is filled when it or its mirror has a nonzero
-// weight sum (sums of positive weights, never -0), tested on the bits.
-__global__ void k_grid_mask(int n, const double *__restrict__ acc_w, uint8_t *__restrict__ mask) {
-    const int64_t cells = (int64_t)n * n;
-    const unsigned long long *wb = (const unsigned long long *)acc_w;
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < cells;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        const int ix = (int)(p % n), iy = (int)(p / n);
-        const int mx = ix == 0 ? 0 : n - ix, my = iy == 0 ? 0 : n - iy;
-        const int64_t pm = (int64_t)my * n + mx;
-        mask[p] = (ix != n / 2 && iy != n / 2 && (wb[p] != 0ull || wb[pm] != 0ull)) ? 1 : 0;
+    grid[p] = g;
+    wsum[p] = w;
+    mask[p] = on;
+    if (iy != 0 && iy != n / 2) {
+        grid[pm] = make_float2(g.x, -g.y);
+        wsum[pm] = w;
+        mask[pm] = on;
     }
 }
 
 struct PlanBufs {
-    uint32_t *keys, *k2, *v2, *k3, *v3, *rhist, *roffs;
     uint32_t *s_idx;      // sorted original indices
     float2 *s_uv;         // sorted positions
-    int64_t n_vis;
-    int ntiles, nchunks;
+    int ntiles;
 };
 
 bool plan_bufs(abs_ctx *ctx, const GridGeom &G, int64_t n_vis, PlanBufs &b) {
     b.ntiles = G.tt * G.tt;
-    b.n_vis = n_vis;
     const int64_t nv = n_vis > 0 ? n_vis : 1;
-    b.nchunks = (int)cdiv(nv, RT);
-    b.keys = (uint32_t *)workspace(ctx, "plan.keys", sizeof(uint32_t) * nv);
-    b.k2 = (uint32_t *)workspace(ctx, "plan.k2", sizeof(uint32_t) * nv);
-    b.v2 = (uint32_t *)workspace(ctx, "plan.v2", sizeof(uint32_t) * nv);
-    b.k3 = b.v3 = nullptr;   // the middle pass of a three-pass sort only
-    b.rhist = (uint32_t *)workspace(ctx, "plan.rhist", sizeof(uint32_t) * ((size_t)1 << DMAX) * b.nchunks);
-    b.roffs = (uint32_t *)workspace(ctx, "plan.roffs", sizeof(uint32_t) * ((size_t)1 << DMAX) * b.nchunks);
     b.s_idx = (uint32_t *)workspace(ctx, "plan.s_idx", sizeof(uint32_t) * nv);
     b.s_uv = (float2 *)workspace(ctx, "plan.s_uv", sizeof(float2) * nv);
-    return b.keys && b.k2 && b.v2 && b.rhist && b.roffs && b.s_idx && b.s_uv;
+    return b.s_idx && b.s_uv;
 }
 
 }  // namespace
-
-// Exclusive scan of len uint32 values (2 kernels; bsum needs cdiv(len, 4096) + 1 entries).
-bool scan_u32(abs_ctx *ctx, const uint32_t *in, int64_t len, uint32_t *out, uint32_t *bsum) {
-    unsigned *ticket = (unsigned *)workspace_zeroed(ctx, "scan.ticket", sizeof(unsigned));
-    if (!ticket) return false;
-    const int nblk = (int)cdiv(len, 4096);
-    if (nblk == 0) return true;
-    k_scan<<<nblk, 1024, 0, ctx->stream>>>(in, len, out, bsum, ticket, nullptr);
-    k_scan_add<<<(int)cdiv(len, 256), 256, 0, ctx->stream>>>(out, len, bsum);
-    return true;
-}
 
 // The key of an invalid visibility: above every (tile, cell) key.
 static uint32_t plan_key_none(const PlanBufs &b) { return (uint32_t)b.ntiles << CB; }
@@ -746,41 +715,38 @@ abs_status launch_grid_plan(abs_ctx *ctx, const Setup &s, int64_t n_vis, const f
     int bits = 1;
     while (((uint64_t)1 << bits) <= (uint64_t)key_none) ++bits;
     const int passes = (bits + DMAX - 1) / DMAX;
-    const int dw = (bits + passes - 1) / passes;
-    if (passes == 3) {
-        b.k3 = (uint32_t *)workspace(ctx, "plan.k3", sizeof(uint32_t) * n_vis);
-        b.v3 = (uint32_t *)workspace(ctx, "plan.v3", sizeof(uint32_t) * n_vis);
-        if (!b.k3 || !b.v3) return fail(ctx, ABS_ERR_OOM, "grid plan workspace");
-    }
-    // one pass: the digit is the key itself, so exactly key_none + 1 bins
-    const int nbins0 = passes == 1 ? (int)key_none + 1 : 1 << dw;
-    const int64_t rlen = (int64_t)std::max(nbins0, 1 << dw) * b.nchunks;
-    uint32_t *bsum = (uint32_t *)workspace(ctx, "plan.bsum", sizeof(uint32_t) * (cdiv(rlen, 4096) + 1));
-    unsigned *ticket = (unsigned *)workspace_zeroed(ctx, "scan.ticket", sizeof(unsigned));
-    if (!bsum || !ticket) return fail(ctx, ABS_ERR_OOM, "grid plan workspace");
+    const int dw = (bits + passes - 1) / passes, nb = 1 << dw;
+    // two slices an SM, of whole rows of a CTA
+    const int64_t per_slice = cdiv(cdiv(n_vis, 2 * ctx->sm_count), ST_T) * ST_T;
+    const int slices = (int)cdiv(n_vis, per_slice);
+    uint32_t *hist = (uint32_t *)workspace(ctx, "plan.hist", sizeof(uint32_t) * ((size_t)slices * nb + nb));
+    // the passes alternate between the scratch and the sorted arrays, ending in the latter; the keys
+    // between two arrays of their own
+    const bool two = passes > 1, three = passes > 2;
+    float2 *t_uv = two ? (float2 *)workspace(ctx, "plan.t_uv", sizeof(float2) * n_vis) : nullptr;
+    uint32_t *t_idx = two ? (uint32_t *)workspace(ctx, "plan.t_idx", sizeof(uint32_t) * n_vis) : nullptr;
+    uint32_t *k1 = two ? (uint32_t *)workspace(ctx, "plan.k1", sizeof(uint32_t) * n_vis) : nullptr;
+    uint32_t *k2 = three ? (uint32_t *)workspace(ctx, "plan.k2", sizeof(uint32_t) * n_vis) : nullptr;
+    if (!hist || (two && (!t_uv || !t_idx || !k1)) || (three && !k2)) return fail(ctx, ABS_ERR_OOM, "grid plan workspace");
+    uint32_t *total = hist + (size_t)slices * nb;
     cudaStream_t st = ctx->stream;
     StageTimer timer(ctx, "grid_plan");
-    const size_t ssmem0 = scatter_smem(nbins0), ssmem = scatter_smem(1 << dw);
-    allow_smem(k_radix_scatter, std::max(ssmem0, ssmem));
-    const uint32_t dmask = passes == 1 ? 0xffffffffu : (uint32_t)((1 << dw) - 1);
-    k_plan_keys<<<b.nchunks, KT, 0, st>>>(G, n_vis, (const float2 *)d_uv, b.keys, key_none, nbins0, dmask,
-                                          b.nchunks, b.rhist);
-    // stable sort of (key, index): keys -> (k2, v2) [-> (k3, v3)] -> (s_idx, s_uv).
-    // Every scan clears the histogram it read, and every scatter but the last
-    // counts the next pass's histogram into it.
-    const uint32_t *ki = b.keys, *vi = nullptr;
+    const size_t smem = sort_smem(nb);
+    const float2 *uin = (const float2 *)d_uv;
+    const uint32_t *iin = nullptr, *kin = nullptr;
     for (int ps = 0; ps < passes; ++ps) {
-        const bool last = ps == passes - 1;
-        const int nbins = ps == 0 ? nbins0 : 1 << dw;
-        const int64_t len = (int64_t)nbins * b.nchunks;
-        k_scan<<<(int)cdiv(len, 4096), 1024, 0, st>>>(b.rhist, len, b.roffs, bsum, ticket,
-                                                      last ? nullptr : b.rhist);
-        uint32_t *ko = ps % 2 == 0 ? b.k2 : b.k3, *vo = ps % 2 == 0 ? b.v2 : b.v3;
-        k_radix_scatter<<<b.nchunks, ST_T, ps == 0 ? ssmem0 : ssmem, st>>>(
-            ki, vi, n_vis, dw * ps, nbins, dmask, b.nchunks, b.roffs, bsum, last ? nullptr : ko,
-            last ? b.s_idx : vo, (const float2 *)d_uv, last ? b.s_uv : nullptr, dw, last ? nullptr : b.rhist);
-        ki = ko;
-        vi = vo;
+        const bool first = ps == 0, last = ps == passes - 1, to_out = (passes - 1 - ps) % 2 == 0;
+        float2 *uo = to_out ? b.s_uv : t_uv;
+        uint32_t *io = to_out ? b.s_idx : t_idx, *ko = last ? nullptr : first ? k1 : k2;
+        if (first) k_plan_hist<true><<<slices, ST_T, 0, st>>>(G, n_vis, per_slice, uin, nullptr, key_none, dw * ps, dw, hist);
+        else k_plan_hist<false><<<slices, ST_T, 0, st>>>(G, n_vis, per_slice, nullptr, kin, key_none, dw * ps, dw, hist);
+        k_plan_offsets<<<(int)cdiv(nb, 8), 256, 0, st>>>(nb, slices, hist, total);
+        const ScatterFn scatter = scatter_of(dw, first, last);
+        allow_smem(scatter, smem);
+        scatter<<<slices, ST_T, smem, st>>>(G, n_vis, per_slice, uin, iin, kin, key_none, dw * ps, hist, total, uo, io, ko);
+        uin = uo;
+        iin = io;
+        kin = ko;
     }
     return check_launch(ctx, "grid plan");
 }
@@ -827,19 +793,11 @@ abs_status launch_grid_accumulate(abs_ctx *ctx, const Setup &s, int64_t n_vis, c
         else
             run(k_grid<GW_SUM>);
     }
-    if (!d_grid && !d_wsum) {   // estimate path: the mask alone, if asked for
-        if (d_mask) {
-            StageTimer timer(ctx, "grid_mask");
-            const int fb = (int)std::min<int64_t>(cdiv(cells, 256), ctx->sm_count * 8);
-            k_grid_mask<<<fb, 256, 0, st>>>(s.n, acc + 2 * cells, d_mask);
-        }
-        return check_launch(ctx, "grid accumulate");
-    }
+    if (estimate) return check_launch(ctx, "grid accumulate");   // read from the accumulators
     {
         StageTimer timer(ctx, "grid_finalize");
-        const int fb = (int)std::min<int64_t>(cdiv(cells, 256), ctx->sm_count * 8);
-        k_grid_finalize<<<fb, 256, 0, st>>>(s.n, acc, acc + cells, acc + 2 * cells,
-                                            (float2 *)d_grid, d_wsum, d_mask);
+        k_grid_finalize<<<dim3((unsigned)cdiv(s.n, 256), s.n / 2 + 1), 256, 0, st>>>(s.n, acc, acc + cells, acc + 2 * cells,
+                                                                                     (float2 *)d_grid, d_wsum, d_mask);
     }
     return check_launch(ctx, "grid accumulate");
 }
