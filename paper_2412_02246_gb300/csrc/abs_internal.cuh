@@ -233,8 +233,6 @@ abs_status launch_triple_sums(abs_ctx *ctx, const Setup &s, const float *d_field
 // the fields already.
 abs_status launch_triple_tc(abs_ctx *ctx, const Setup &s, const float *d_fields,
                             int32_t n_trip, const int32_t *d_ijk, double *d_sum);
-// Uploads the ring geometry of a derived setup (d_ring_geom); false if it cannot be allocated.
-bool make_ring_geometry(Setup &s);
 // Ring tables (cell lists, byte map) from d_mask, or, with d_accw given, from
 // the FP64 weight sums before the mirror (a cell is filled when it or its
 // mirror has a nonzero sum), then exact counts (d_count may be NULL) and, if

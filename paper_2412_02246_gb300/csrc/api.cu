@@ -357,7 +357,7 @@ const Setup *get_setup(abs_ctx *ctx, const abs_config *cfg, abs_status &st) {
     s->d_ijk = upload(s->ijk);
     s->d_tw = upload(tw);
     s->d_Rm = upload(std::vector<int32_t>(s->Rm.begin(), s->Rm.end()));
-    if (!make_ring_geometry(*s) || !s->d_q || !s->d_lat_off || !s->d_ijk || !s->d_tw || !s->d_Rm) {
+    if (!s->d_q || !s->d_lat_off || !s->d_ijk || !s->d_tw || !s->d_Rm) {
         free_setup(*s);
         st = fail(ctx, ABS_ERR_OOM, "setup tables");
         return nullptr;

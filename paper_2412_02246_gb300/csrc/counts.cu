@@ -636,40 +636,8 @@ int count_warps(int nb) {
     return (int)std::min<size_t>(CT / 32, (96 * 1024) / ((size_t)(nb + 1) * 32 * 2));
 }
 
-// Ring tables of the filled set; with ia the tables and work items of the counts too.
-abs_status ring_tables(abs_ctx *ctx, const Setup &s, const uint8_t *d_mask, const double *d_accw, RingTables &T,
-                       double *d_ellbar, ItemArgs *ia) {
-    const CountGeom G = cgeom(s);
-    const int64_t U = std::max(G.nU, 1), O = std::max(G.nO, 1), mb = map_bytes_of(G);
-    short2 *lists = (short2 *)workspace(ctx, "ring.lists", sizeof(short2) * 2 * U + sizeof(uint32_t) * O + O);
-    // the filled map, the hole table, the counters: cleared together
-    const int64_t cb = mb + sizeof(unsigned long long) * s.nb * s.nb + sizeof(int32_t) * 3 * s.nb + sizeof(int) * 8;
-    uint8_t *clr = (uint8_t *)workspace(ctx, "ring.maps", cb);
-    if (!lists || !clr) return fail(ctx, ABS_ERR_OOM, "ring table workspace");
-    T.F = lists;
-    T.H = lists + U;
-    T.HO = (uint32_t *)(lists + 2 * U);
-    T.nf = (uint8_t *)(T.HO + O);
-    T.mapF = clr;
-    T.fix = (unsigned long long *)(clr + mb);
-    T.cnt = (int32_t *)(T.fix + (size_t)s.nb * s.nb);
-    T.ctl = (int *)(T.cnt + 3 * s.nb);
-    StageTimer timer(ctx, "ring_lists");
-    cudaStream_t st = ctx->stream;
-    cudaMemsetAsync(clr, 0, cb, st);
-    const int ub = (int)cdiv(U, 256), ob = (int)cdiv(O, 256);
-    k_ring_cells<<<ub + ob, 256, 0, st>>>(G, ub, d_mask, (const unsigned long long *)d_accw, T);
-    const ItemArgs none{};
-    // blocks: a ring each for the mean l and the tables, and enough warps for the pairs (32 each)
-    const int np = s.nb * s.nb;
-    const int blocks = ia ? std::max<int>(s.nb, std::min<int>((int)cdiv(3 * np, 256), 2 * ctx->sm_count)) : s.nb;
-    k_ring_finish<<<blocks, 256, 0, st>>>(G, s.du, T, d_ellbar, ia ? *ia : none);
-    return check_launch(ctx, "ring lists");
-}
-
-}  // namespace
-
-// The ring geometry's device tables (one allocation) and the counts' item capacities.
+// The ring geometry's device tables (one allocation) and the counts' item capacities, made on the first
+// call that counts or averages over a ring.
 bool make_ring_geometry(Setup &s) {
     const int nb = s.nb, R = s.R, W = 2 * R + 1;
     const int64_t nU = s.up_off.back();
@@ -733,15 +701,52 @@ bool make_ring_geometry(Setup &s) {
     }
     if (cudaMemcpy(s.d_ring_geom, host.data(), total, cudaMemcpyHostToDevice) != cudaSuccess) {
         cudaGetLastError();
+        cudaFree(s.d_ring_geom);
+        s.d_ring_geom = nullptr;
         return false;
     }
     return true;
 }
 
+// Ring tables of the filled set; with ia the tables and work items of the counts too.
+abs_status ring_tables(abs_ctx *ctx, const Setup &s, const uint8_t *d_mask, const double *d_accw, RingTables &T,
+                       double *d_ellbar, ItemArgs *ia) {
+    if (!s.d_ring_geom && !make_ring_geometry(const_cast<Setup &>(s))) return fail(ctx, ABS_ERR_OOM, "ring geometry");
+    const CountGeom G = cgeom(s);
+    const int64_t U = std::max(G.nU, 1), O = std::max(G.nO, 1), mb = map_bytes_of(G);
+    short2 *lists = (short2 *)workspace(ctx, "ring.lists", sizeof(short2) * 2 * U + sizeof(uint32_t) * O + O);
+    // the filled map, the hole table, the counters: cleared together
+    const int64_t cb = mb + sizeof(unsigned long long) * s.nb * s.nb + sizeof(int32_t) * 3 * s.nb + sizeof(int) * 8;
+    uint8_t *clr = (uint8_t *)workspace(ctx, "ring.maps", cb);
+    if (!lists || !clr) return fail(ctx, ABS_ERR_OOM, "ring table workspace");
+    T.F = lists;
+    T.H = lists + U;
+    T.HO = (uint32_t *)(lists + 2 * U);
+    T.nf = (uint8_t *)(T.HO + O);
+    T.mapF = clr;
+    T.fix = (unsigned long long *)(clr + mb);
+    T.cnt = (int32_t *)(T.fix + (size_t)s.nb * s.nb);
+    T.ctl = (int *)(T.cnt + 3 * s.nb);
+    StageTimer timer(ctx, "ring_lists");
+    cudaStream_t st = ctx->stream;
+    cudaMemsetAsync(clr, 0, cb, st);
+    const int ub = (int)cdiv(U, 256), ob = (int)cdiv(O, 256);
+    k_ring_cells<<<ub + ob, 256, 0, st>>>(G, ub, d_mask, (const unsigned long long *)d_accw, T);
+    const ItemArgs none{};
+    // blocks: a ring each for the mean l and the tables, and enough warps for the pairs (32 each)
+    const int np = s.nb * s.nb;
+    const int blocks = ia ? std::max<int>(s.nb, std::min<int>((int)cdiv(3 * np, 256), 2 * ctx->sm_count)) : s.nb;
+    k_ring_finish<<<blocks, 256, 0, st>>>(G, s.du, T, d_ellbar, ia ? *ia : none);
+    return check_launch(ctx, "ring lists");
+}
+
+}  // namespace
+
 abs_status launch_counts(abs_ctx *ctx, const Setup &s, const uint8_t *d_mask, int32_t n_trip,
                          const int32_t *d_ijk, int64_t *d_count, double *d_ellbar, const double *d_accw) {
     RingTables T;
     if (n_trip == 0 || !d_count) return ring_tables(ctx, s, d_mask, d_accw, T, d_ellbar, nullptr);
+    if (!s.d_ring_geom && !make_ring_geometry(const_cast<Setup &>(s))) return fail(ctx, ABS_ERR_OOM, "ring geometry");
     const CountGeom G = cgeom(s);
     const int hs = s.nb + 1;
     const int64_t map_bytes = map_bytes_of(G);
