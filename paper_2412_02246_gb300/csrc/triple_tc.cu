@@ -190,19 +190,33 @@ __host__ __device__ constexpr uint32_t make_idesc(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// D (tensor memory) += A (tensor memory) x B (shared-memory descriptor)^T.
+// The issuing warps run converged, every value the same in all lanes (uni), and only the issue itself is
+// one lane's (elect.sync, always the same lane): so the compiler keeps the MMA's operands in uniform
+// registers, where the instruction takes them.  Issued from inside an `if (lane == 0)`, each MMA
+// waited for its operands to be moved there: 83 cycles apart instead of the tensor pipe's rate.
+constexpr unsigned FULL = 0xffffffffu;
+template <class T>
+__device__ __forceinline__ T uni(T x) {
+    return __shfl_sync(FULL, x, 0);
+}
+
+// D (tensor memory) += A (tensor memory) x B (shared-memory descriptor)^T, issued by one lane of the warp.
 __device__ __forceinline__ void mma_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t b, uint32_t idesc,
                                        uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
+        "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n"
         ::"r"(tmem_d), "r"(tmem_a), "l"(b), "r"(idesc), "r"(accumulate));
 }
 
 __device__ __forceinline__ void mma_commit(uint32_t mbar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
-                 ::"r"(mbar) : "memory");
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n"
+        ::"r"(mbar) : "memory");
 }
 
 __device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t count) {
@@ -334,7 +348,7 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
     __shared__ int64_t blk_out[FQ][MAXBLK];
     // stages on a 1024-byte boundary (the 128-byte swizzle's atom); the launch adds 1 KB of slack
     uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uni((int)(threadIdx.x >> 5)), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         abort_s = 0;
         for (int s = 0; s < G.n_stages; ++s) {
@@ -357,7 +371,7 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    const uint32_t tmem = tmem_holder;
+    const uint32_t tmem = uni(tmem_holder);
 
     // role state that lives across items
     int st = 0, su = 0;      // stage and its use (loader, formers and issuer walk the same sequence)
@@ -375,10 +389,10 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
         // item comes from the launch's work counter (items in pixel-range order, so the
         // CTAs work on neighbouring ranges at any time and share them in L2)
         __syncthreads();
-        if (abort_s) break;
+        if (__any_sync(FULL, abort_s)) break;
         if (threadIdx.x == 0) item_s = atomicAdd(next_item, 1);
         __syncthreads();
-        const int e = item_s;
+        const int e = uni(item_s);
         if (e >= G.n_items) break;
         const int set_id = e % G.n_sets;
         const int64_t p0 = (int64_t)(e / G.n_sets) * G.per_item;
@@ -440,78 +454,77 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
                 }
             }
         } else if (warp <= NISS) {
-            // ---------------- MMA issue (one thread a warp): groups of DRAIN chunks into alternating
+            // ---------------- MMA issue (the whole warp, one lane's instruction): groups of DRAIN chunks into alternating
             // regions.  Every issuer walks every chunk (waits and commits alike, so that the
             // barriers count NISS arrivals a phase) and issues the MMAs of its own tiles.  The
             // per-chunk path is kept short (tile constants in registers, the stage's descriptor
             // advanced by addition): the tensor pipe idles while an issuer is between chunks.
             const int iss = warp - 1;
-            if (lane == 0) {
-                uint32_t idesc_t[MAX_TILES], col_t[MAX_TILES], rows_t[MAX_TILES];
+            const int ntiles = uni(S.ntiles);
+            uint32_t idesc_t[MAX_TILES], col_t[MAX_TILES], rows_t[MAX_TILES];
+#pragma unroll
+            for (int t = 0; t < MAX_TILES; ++t) {
+                idesc_t[t] = uni(t < ntiles ? make_idesc(TM, t_n[t]) : 0u);
+                col_t[t] = uni(t < ntiles ? (uint32_t)t_col[t] : 0u);
+                rows_t[t] = uni(t < ntiles ? (uint32_t)(t_ilo[t] - S.b_lo) * 8u : 0u);
+            }
+            const uint32_t cols = uni((uint32_t)region_cols);
+            const uint64_t d_stage = (uint64_t)(G.stage_bytes >> 4), d_lo = (uint64_t)uni((uint32_t)b_bytes >> 4);
+            const uint64_t d_base = desc_sw128(uni(smem_u32(smem)));
+            uint64_t d_cur = d_base + (uint64_t)st * d_stage;   // this chunk's stage, B hi plane
+            int gc = 0;                                          // chunk in the group
+            auto wait = [&](const uint64_t *bar, int parity) {
+                return __all_sync(FULL, mbar_wait(smem_u32(bar), (uint32_t)parity, &abort_s)) != 0;
+            };
+            for (int c = 0; c < nchunks; ++c) {
+                const uint32_t region = (uint32_t)(NABUF * A_COLS) + (grp & 1) * cols;
+                bool ok = true;
+                if (gc == 0 && grp >= 2) {   // the group before last in this region has been drained
+                    ok = wait(&d_empty[grp & 1], ((grp >> 1) - 1) & 1);
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                }
+                ok = ok && wait(&full[st], su & 1);
+                const uint32_t a_slot = tmem + (uint32_t)((cg & (ASLOTS - 1)) * MAX_TILES * A_COLS);
+                const uint32_t first = gc > 0 ? 1u : 0u;
 #pragma unroll
                 for (int t = 0; t < MAX_TILES; ++t) {
-                    idesc_t[t] = t < S.ntiles ? make_idesc(TM, t_n[t]) : 0u;
-                    col_t[t] = t < S.ntiles ? (uint32_t)t_col[t] : 0u;
-                    rows_t[t] = t < S.ntiles ? (uint32_t)(t_ilo[t] - S.b_lo) * 8u : 0u;
-                }
-                const uint64_t d_stage = (uint64_t)(G.stage_bytes >> 4), d_lo = (uint64_t)(b_bytes >> 4);
-                const uint64_t d_base = desc_sw128(smem_u32(smem));
-                uint64_t d_cur = d_base + (uint64_t)st * d_stage;   // this chunk's stage, B hi plane
-                int gc = 0;                                          // chunk in the group
-                for (int c = 0; c < nchunks && !abort_s; ++c) {
-                    const uint32_t region = (uint32_t)(NABUF * A_COLS + (grp & 1) * region_cols);
-                    if (gc == 0 && grp >= 2) {   // the group before last in this region has been drained
-                        if (!mbar_wait(smem_u32(&d_empty[grp & 1]), (uint32_t)(((grp >> 1) - 1) & 1), &abort_s)) {
-                            abort_s = 1;
-                            break;
-                        }
-                        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    }
-                    if (!mbar_wait(smem_u32(&full[st]), (uint32_t)(su & 1), &abort_s)) {
-                        abort_s = 1;
-                        break;
-                    }
-                    const uint32_t a_slot = tmem + (uint32_t)((cg & (ASLOTS - 1)) * MAX_TILES * A_COLS);
-                    const uint32_t first = gc > 0 ? 1u : 0u;
+                    if (t >= ntiles || !ok) break;
+                    if (t % NISS != iss) continue;
+                    // this tile's A buffers, formed ahead
+                    ok = wait(&a_full[(cg & (ASLOTS - 1)) * MAX_TILES + t], (cg / ASLOTS) & 1);
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                    // a tile's rows and a K-step move only the descriptors' start-address field
+                    // (16-byte units: 8 per ring row, 2 per 16 pixels)
+                    const uint32_t acc = tmem + region + col_t[t];
+                    const uint32_t a_hi = a_slot + (uint32_t)(t * A_COLS), a_lo = a_hi + 32;
+                    const uint64_t dh0 = d_cur + rows_t[t], dl0 = dh0 + d_lo;
 #pragma unroll
-                    for (int t = 0; t < MAX_TILES; ++t) {
-                        if (t >= S.ntiles) break;
-                        if (t % NISS != iss) continue;
-                        // this tile's A buffers, formed ahead
-                        if (!mbar_wait(smem_u32(&a_full[(cg & (ASLOTS - 1)) * MAX_TILES + t]),
-                                       (uint32_t)((cg / ASLOTS) & 1), &abort_s)) {
-                            abort_s = 1;
-                            break;
-                        }
-                        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                        // a tile's rows and a K-step move only the descriptors' start-address field
-                        // (16-byte units: 8 per ring row, 2 per 16 pixels)
-                        const uint32_t acc = tmem + region + col_t[t];
-                        const uint32_t a_hi = a_slot + (uint32_t)(t * A_COLS), a_lo = a_hi + 32;
-                        const uint64_t dh0 = d_cur + rows_t[t], dl0 = dh0 + d_lo;
-#pragma unroll
-                        for (int ks = 0; ks < KC / 16; ++ks) {
-                            mma_ts(acc, a_hi + 8u * ks, dh0 + 2u * ks, idesc_t[t], ks > 0 ? 1u : first);
-                            mma_ts(acc, a_hi + 8u * ks, dl0 + 2u * ks, idesc_t[t], 1u);
-                            mma_ts(acc, a_lo + 8u * ks, dh0 + 2u * ks, idesc_t[t], 1u);
-                        }
+                    for (int ks = 0; ks < KC / 16; ++ks) {
+                        mma_ts(acc, a_hi + 8u * ks, dh0 + 2u * ks, idesc_t[t], ks > 0 ? 1u : first);
+                        mma_ts(acc, a_hi + 8u * ks, dl0 + 2u * ks, idesc_t[t], 1u);
+                        mma_ts(acc, a_lo + 8u * ks, dh0 + 2u * ks, idesc_t[t], 1u);
                     }
-                    // one commit a chunk: its MMAs done frees the stage and the chunk's A buffers
-                    mma_commit(smem_u32(&done[st]));
-                    ++cg;
-                    if (++st == G.n_stages) {
-                        st = 0;
-                        ++su;
-                        d_cur = d_base;
-                    } else {
-                        d_cur += d_stage;
-                    }
-                    if (gc == DRAIN - 1 || c == nchunks - 1) {   // the group is complete: the formers drain it
-                        mma_commit(smem_u32(&d_full[grp & 1]));
-                        ++grp;
-                    }
-                    if (++gc == DRAIN) gc = 0;
                 }
+                if (!ok) {
+                    abort_s = 1;
+                    break;
+                }
+                // one commit a chunk: its MMAs done frees the stage and the chunk's A buffers
+                mma_commit(smem_u32(&done[st]));
+                ++cg;
+                if (++st == G.n_stages) {
+                    st = 0;
+                    ++su;
+                    d_cur = d_base;
+                } else {
+                    d_cur += d_stage;
+                }
+                if (gc == DRAIN - 1 || c == nchunks - 1) {   // the group is complete: the formers drain it
+                    mma_commit(smem_u32(&d_full[grp & 1]));
+                    ++grp;
+                }
+                if (++gc == DRAIN) gc = 0;
             }
         } else {
             // ---------------- formers; after the first chunk of each group they drain the group before
@@ -656,7 +669,7 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
                 if (!mbar_drain(smem_u32(&full[s]), (uint32_t)((uses - 1) & 1))) break;
             }
         }
-        if (warp >= 1 && warp <= NISS && lane == 0) {
+        if (warp >= 1 && warp <= NISS) {
             // every MMA the issuers issued is done once a fresh commit of each arrives
             mma_commit(smem_u32(&fin));
             mbar_drain(smem_u32(&fin), 0u);
