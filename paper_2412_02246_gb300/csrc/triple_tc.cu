@@ -322,10 +322,12 @@ __device__ __forceinline__ void tmem_st(uint32_t ta, const uint32_t (&v)[8]) {
 // A pair of FP32 values as BF16 hi parts and BF16 residuals, each packed (first value low).
 __device__ __forceinline__ void split2(float2 v, uint32_t &hi, uint32_t &lo) {
     const __nv_bfloat162 h = __float22bfloat162_rn(v);
-    const float2 hf = __bfloat1622float2(h);
+    hi = *(const uint32_t *)&h;
+    // the two hi parts as FP32: a shift and a mask (two byte permutes, which the library's conversion
+    // takes, both go to the pipe that already does the packing)
+    const float2 hf = make_float2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u));
     const float2 r = __ffma2_rn(hf, make_float2(-1.f, -1.f), v);   // v - hi, exact in FP32
     const __nv_bfloat162 l = __float22bfloat162_rn(r);
-    hi = *(const uint32_t *)&h;
     lo = *(const uint32_t *)&l;
 }
 
@@ -533,30 +535,33 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
             const int row = 32 * q + lane;
             const uint32_t lane_base = tmem + ((uint32_t)(32 * q) << 16);
             const int nb_h = n_blk[h];
-            // this thread's rows of the set's tiles: offsets of D_j and D_k in an F window
+            // this thread's rows of the set's tiles: offsets of D_j and D_k in an F window (a row the tile
+            // does not have forms the window's first ring; its sums are never read)
             uint32_t rel_j[MAX_TILES], rel_k[MAX_TILES];
-            bool row_ok[MAX_TILES];
 #pragma unroll
             for (int t = 0; t < MAX_TILES; ++t) {
                 const short2 jk = t < S.ntiles ? rows_s[t][row] : make_short2(-1, -1);
-                row_ok[t] = jk.x >= 0;
-                rel_j[t] = row_ok[t] ? frow_rel(jk.x, S.f_lo, (h * FPX) / 4) : 0u;
-                rel_k[t] = row_ok[t] ? frow_rel(jk.y, S.f_lo, (h * FPX) / 4) : 0u;
+                rel_j[t] = jk.x >= 0 ? frow_rel(jk.x, S.f_lo, (h * FPX) / 4) : 0u;
+                rel_k[t] = jk.x >= 0 ? frow_rel(jk.y, S.f_lo, (h * FPX) / 4) : 0u;
             }
             int gdrained = grp;                       // this item's first group
             bool fail_f = false;
+            // a barrier test takes over 100 cycles to answer, so the next chunk's two are asked for before the
+            // end of this one: the copies have landed; the MMAs that read the next chunk's A slot are done
+            bool full_ok = false, done_ok = false;
             // chunk c is formed; after the first chunk of a group (and after the last chunk) the group
             // before is drained: its accumulation region is added into accl and released
             for (int c = 0; c <= nchunks && !fail_f; ++c) {
                 if (c < nchunks) {
-                    if (!mbar_wait(smem_u32(&full[st]), (uint32_t)(su & 1), &abort_s)) {
+                    if (!full_ok && !mbar_wait(smem_u32(&full[st]), (uint32_t)(su & 1), &abort_s)) {
                         fail_f = true;
                         break;
                     }
                     // the F window
                     const uint8_t *F = smem + (size_t)st * G.stage_bytes + 2 * b_bytes;
                     // the A buffers of this chunk's pair were read by the MMAs of chunk cg - 2
-                    if (cg >= ASLOTS && !mbar_wait(smem_u32(&done[hst[0]]), (uint32_t)(hsu[0] & 1), &abort_s)) {
+                    if (!done_ok && cg >= ASLOTS &&
+                        !mbar_wait(smem_u32(&done[hst[0]]), (uint32_t)(hsu[0] & 1), &abort_s)) {
                         fail_f = true;
                         break;
                     }
@@ -567,6 +572,7 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
                     }
                     hst[ASLOTS - 1] = st;
                     hsu[ASLOTS - 1] = su;
+                    const int nst = st + 1 == G.n_stages ? 0 : st + 1, nsu = st + 1 == G.n_stages ? su + 1 : su;
                     const uint32_t Fs = after_wait(smem_u32(F));
 #pragma unroll
                     for (int t = 0; t < MAX_TILES; ++t) {
@@ -578,22 +584,21 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
 #pragma unroll
                         for (int part = 0; part < FPX / 16; ++part) {
                             uint32_t hi[8], lo[8];
-                            if (row_ok[t]) {
 #pragma unroll
-                                for (int cc = 0; cc < 4; ++cc) {
-                                    const uint32_t w = (uint32_t)(4 * part + cc) << 4;
-                                    const float4 x = lds128(pj ^ w), y = lds128(pk ^ w);
-                                    split2(__fmul2_rn(make_float2(x.x, x.y), make_float2(y.x, y.y)), hi[2 * cc],
-                                           lo[2 * cc]);
-                                    split2(__fmul2_rn(make_float2(x.z, x.w), make_float2(y.z, y.w)), hi[2 * cc + 1],
-                                           lo[2 * cc + 1]);
-                                }
-                            } else {
-#pragma unroll
-                                for (int cc = 0; cc < 8; ++cc) hi[cc] = lo[cc] = 0u;
+                            for (int cc = 0; cc < 4; ++cc) {
+                                const uint32_t w = (uint32_t)(4 * part + cc) << 4;
+                                const float4 x = lds128(pj ^ w), y = lds128(pk ^ w);
+                                split2(__fmul2_rn(make_float2(x.x, x.y), make_float2(y.x, y.y)), hi[2 * cc],
+                                       lo[2 * cc]);
+                                split2(__fmul2_rn(make_float2(x.z, x.w), make_float2(y.z, y.w)), hi[2 * cc + 1],
+                                       lo[2 * cc + 1]);
                             }
                             tmem_st(ta + 8u * part, hi);
                             tmem_st(ta + 32u + 8u * part, lo);
+                        }
+                        if (t == S.ntiles - 1 && c + 1 < nchunks) {
+                            full_ok = mbar_test(smem_u32(&full[nst]), (uint32_t)(nsu & 1));
+                            done_ok = cg + 1 >= ASLOTS && mbar_test(smem_u32(&done[hst[0]]), (uint32_t)(hsu[0] & 1));
                         }
                         // tile t's A buffers are complete: its issuer may start while the next is formed
                         asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
@@ -606,11 +611,8 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
                         for (int t = S.ntiles; t < MAX_TILES; ++t)
                             mbar_arrive(smem_u32(&a_full[(cg & (ASLOTS - 1)) * MAX_TILES + t]));
                     ++cg;
-                    if (fail_f) break;
-                    if (++st == G.n_stages) {
-                        st = 0;
-                        ++su;
-                    }
+                    st = nst;
+                    su = nsu;
                 }
                 if (c == nchunks || (c % DRAIN == 0 && c > 0)) {
                     const int g = gdrained;
