@@ -44,6 +44,11 @@ namespace {
 
 constexpr int MAXRAD = 16;
 constexpr int MAX_RADIX = 16;   // largest radix of a pass (composite radices up to it, see Dft)
+// The transform kernels come in two forms, for plans of radices up to LOW_RADIX and for the others: the
+// radix-16 butterfly in double-float sets the registers of a kernel that holds it (208 a thread, eight
+// warps an SM), and the plans of most sizes (N = 288 = 8 6 6, 576 = 9 8 8) never take it.
+constexpr int LOW_RADIX = 9;
+constexpr int DF_BLOCKS = 4;
 __host__ __device__ constexpr int itw_off(int R) { return R * (R - 1) / 2; }
 constexpr int ITW_N = itw_off(MAX_RADIX + 1);
 constexpr int FFT_NT = 128;     // threads per transform CTA
@@ -137,9 +142,6 @@ struct ArithDF {
     __device__ static C half(C a) { return p_half(a); }
     __device__ static C cst(double v) { return pconst(v); }
     __device__ static C mul(C a, C c) { return p_mul(a, c); }
-    __device__ static C twiddle(C v, const float4 *__restrict__ tw, int t) {
-        return c_mul_tw(v, ::absk::ld(__ldg(tw + 2 * t)), ::absk::ld(__ldg(tw + 2 * t + 1)));
-    }
     // w = exp(-2 pi i t / N) as a complex value (re, im) from the table, and v w
     __device__ static C tw_load(const float4 *__restrict__ tw, int t) {
         const float4 c = __ldg(tw + 2 * t), s = __ldg(tw + 2 * t + 1);
@@ -175,11 +177,6 @@ struct ArithF32 {
     __device__ static C half(C a) { return __fmul2_rn(a, f2(0.5f, 0.5f)); }
     __device__ static C cst(double v) { return f2((float)v, (float)v); }
     __device__ static C mul(C a, C c) { return __fmul2_rn(a, c); }
-    // v w = v (c, c) + (v.im, v.re) (-s, s)
-    __device__ static C twiddle(C v, const float4 *__restrict__ tw, int t) {
-        const float4 w = __ldg(tw + t);
-        return __ffma2_rn(f2(v.y, v.x), f2(w.z, w.w), __fmul2_rn(v, f2(w.x, w.y)));
-    }
     __device__ static C tw_load(const float4 *__restrict__ tw, int t) {
         const float4 w = __ldg(tw + t);
         return f2(w.x, w.w);
@@ -353,32 +350,37 @@ __device__ __forceinline__ void stockham_lines(const typename A::E *__restrict__
 }
 
 // One Stockham pass over `lines` transforms of length N stored line-major.
-template <class A>
+template <class A, int MAXR>
 __device__ __forceinline__ void stockham_pass(const typename A::E *__restrict__ in, typename A::E *__restrict__ out,
                                               int N, const FftPass &P, int lines,
                                               const float4 *__restrict__ tw, const float4 *itw) {
     switch (P.R) {
-        case 2: stockham_lines<A, 2>(in, out, N, P, lines, tw, itw); break;
-        case 3: stockham_lines<A, 3>(in, out, N, P, lines, tw, itw); break;
-        case 4: stockham_lines<A, 4>(in, out, N, P, lines, tw, itw); break;
-        case 5: stockham_lines<A, 5>(in, out, N, P, lines, tw, itw); break;
-        case 6: stockham_lines<A, 6>(in, out, N, P, lines, tw, itw); break;
-        case 8: stockham_lines<A, 8>(in, out, N, P, lines, tw, itw); break;
-        case 9: stockham_lines<A, 9>(in, out, N, P, lines, tw, itw); break;
-        case 10: stockham_lines<A, 10>(in, out, N, P, lines, tw, itw); break;
-        case 12: stockham_lines<A, 12>(in, out, N, P, lines, tw, itw); break;
-        case 15: stockham_lines<A, 15>(in, out, N, P, lines, tw, itw); break;
-        default: stockham_lines<A, 16>(in, out, N, P, lines, tw, itw); break;
+        case 2: stockham_lines<A, 2>(in, out, N, P, lines, tw, itw); return;
+        case 3: stockham_lines<A, 3>(in, out, N, P, lines, tw, itw); return;
+        case 4: stockham_lines<A, 4>(in, out, N, P, lines, tw, itw); return;
+        case 5: stockham_lines<A, 5>(in, out, N, P, lines, tw, itw); return;
+        case 6: stockham_lines<A, 6>(in, out, N, P, lines, tw, itw); return;
+        case 8: stockham_lines<A, 8>(in, out, N, P, lines, tw, itw); return;
+        case 9: stockham_lines<A, 9>(in, out, N, P, lines, tw, itw); return;
+        default: break;
+    }
+    if constexpr (MAXR > LOW_RADIX) {
+        switch (P.R) {
+            case 10: stockham_lines<A, 10>(in, out, N, P, lines, tw, itw); return;
+            case 12: stockham_lines<A, 12>(in, out, N, P, lines, tw, itw); return;
+            case 15: stockham_lines<A, 15>(in, out, N, P, lines, tw, itw); return;
+            default: stockham_lines<A, 16>(in, out, N, P, lines, tw, itw); return;
+        }
     }
 }
 
 // Transforms `lines` lines in buffer a (scratch b); returns the buffer holding the result.
-template <class A>
+template <class A, int MAXR>
 __device__ typename A::E *fft_lines(typename A::E *a, typename A::E *b, int lines, const FftPlan &P,
                                     const float4 *__restrict__ tw) {
     for (int s = 0; s < P.nrad; ++s) {
         __syncthreads();
-        stockham_pass<A>(a, b, P.N, P.pass[s], lines, tw, P.itw);
+        stockham_pass<A, MAXR>(a, b, P.N, P.pass[s], lines, tw, P.itw);
         typename A::E *t = a;
         a = b;
         b = t;
@@ -509,8 +511,12 @@ struct GridReal {
 
 // Column pass: one CTA per (block of CB columns x, ring pair), transforming
 // along y the 2R+1 columns |x| <= R that hold ring cells.  W[pair][x + Rmax][N].
-template <class Src, class A>
-__global__ void __launch_bounds__(FFT_NT) k_fft_cols(RingGeom G, const __grid_constant__ FftPlan P, int CB, const int64_t *__restrict__ q,
+// CTAs an SM the registers must leave room for: all that fit for the low-radix double-float kernels.
+template <class A, int MAXR>
+constexpr int fft_min_blocks() { return sizeof(typename A::E) == 16 && MAXR <= LOW_RADIX ? DF_BLOCKS : 1; }
+
+template <class Src, class A, int MAXR>
+__global__ void __launch_bounds__(FFT_NT, fft_min_blocks<A, MAXR>()) k_fft_cols(RingGeom G, const __grid_constant__ FftPlan P, int CB, const int64_t *__restrict__ q,
                                                   const int32_t *__restrict__ Rm, Src src,
                                                   const float4 *__restrict__ tw,
                                                   typename A::E *__restrict__ W) {
@@ -540,7 +546,7 @@ __global__ void __launch_bounds__(FFT_NT) k_fft_cols(RingGeom G, const __grid_co
         // Z = X_a + i X_b
         l0[(size_t)c * G.N + (y < 0 ? y + G.N : y)] = in_a ? A::from_cell(v) : A::times_i(v);
     }
-    E *res = fft_lines<A>(l0, l1, CB, P, tw);
+    E *res = fft_lines<A, MAXR>(l0, l1, CB, P, tw);
     for (int e = threadIdx.x; e < CB * G.N; e += blockDim.x) {
         const int c = e / G.N, x = x0 + c;
         if (x < -Rp || x > Rp) continue;
@@ -704,8 +710,8 @@ __device__ __forceinline__ void row_pass(const RingGeom &G, const FftPlan &P, co
     }
 }
 
-template <class A, class Out>
-__global__ void __launch_bounds__(RowNT<A>::value, RowNT<A>::min_blocks)
+template <class A, class Out, int MAXR>
+__global__ void __launch_bounds__(RowNT<A>::value, RowNT<A>::min_blocks > 1 ? RowNT<A>::min_blocks : fft_min_blocks<A, MAXR>())
     k_fft_rows(RingGeom G, const __grid_constant__ FftPlan P, int RB, uint32_t mag_rb, int LS,
                const int32_t *__restrict__ Rm, const typename A::E *__restrict__ W, const float4 *__restrict__ tw,
                const Out dst_out) {
@@ -730,15 +736,23 @@ __global__ void __launch_bounds__(RowNT<A>::value, RowNT<A>::min_blocks)
         const bool first = s == 0, last = s == P.nrad - 1 && !Out::staged;
         const E *in = buf0 + ((s + 1) & 1) * bstride;   // what pass s - 1 wrote
         E *out = buf0 + (s & 1) * bstride;
-        switch (ps.R) {
 #define ABS_ROW_CASE(RR) \
     case RR: row_pass<A, RR>(G, P, ps, first, last, RB, rb, mag_rb, LS, Rp, py0, src, in, out, tw, dst_out, a, b); break;
-            ABS_ROW_CASE(2) ABS_ROW_CASE(3) ABS_ROW_CASE(4) ABS_ROW_CASE(5) ABS_ROW_CASE(6) ABS_ROW_CASE(8)
-            ABS_ROW_CASE(9) ABS_ROW_CASE(10) ABS_ROW_CASE(12) ABS_ROW_CASE(15)
-            default: row_pass<A, 16>(G, P, ps, first, last, RB, rb, mag_rb, LS, Rp, py0, src, in, out, tw, dst_out, a, b);
-                break;
-#undef ABS_ROW_CASE
+        if (MAXR <= LOW_RADIX || ps.R <= LOW_RADIX) {
+            switch (ps.R) {
+                ABS_ROW_CASE(2) ABS_ROW_CASE(3) ABS_ROW_CASE(4) ABS_ROW_CASE(5) ABS_ROW_CASE(6) ABS_ROW_CASE(8)
+                ABS_ROW_CASE(9)
+                default: break;
+            }
+        } else {
+            if constexpr (MAXR > LOW_RADIX) {
+                switch (ps.R) {
+                    ABS_ROW_CASE(10) ABS_ROW_CASE(12) ABS_ROW_CASE(15) ABS_ROW_CASE(16)
+                    default: break;
+                }
+            }
         }
+#undef ABS_ROW_CASE
     }
     if constexpr (Out::staged) {
         __syncthreads();
@@ -851,6 +865,10 @@ static size_t row_smem(const Setup &s, int RB, int LS, size_t esize, bool staged
 // split-BF16 path, whose triplet products carry a larger error of their own.
 static bool plain_fp32(const Setup &s) { return s.precision == ABS_SPLIT_BF16; }
 
+static bool low_radix(const Setup &s) {
+    return std::all_of(s.radices.begin(), s.radices.end(), [](int r) { return r <= LOW_RADIX; });
+}
+
 FftLaunch fft_launch(const Setup &s, int sm_count) {
     FftLaunch L;
     const bool f32 = plain_fp32(s);
@@ -878,19 +896,20 @@ abs_status run_fft_as(abs_ctx *ctx, const Setup &s, const Src &src, float *d_fie
     const size_t line = sizeof(E) * (size_t)s.N;
     cudaStream_t st = ctx->stream;
     const float4 *tw = A::table(s.d_tw, s.N);
+    const bool low = low_radix(s);
     auto cols = [&](int cb) {
         const size_t sm = line * 2 * cb;
-        allow_smem(k_fft_cols<Src, A>, sm);
-        k_fft_cols<Src, A><<<dim3((unsigned)cdiv(2 * s.R + 1, cb), npairs), FFT_NT, sm, st>>>(G, P, cb, s.d_q,
-                                                                                             s.d_Rm, src, tw, W);
+        const auto kern = low ? k_fft_cols<Src, A, LOW_RADIX> : k_fft_cols<Src, A, MAX_RADIX>;
+        allow_smem(kern, sm);
+        kern<<<dim3((unsigned)cdiv(2 * s.R + 1, cb), npairs), FFT_NT, sm, st>>>(G, P, cb, s.d_q, s.d_Rm, src, tw, W);
     };
     auto rows_to = [&](int rb, const auto &out) {
         using Out = std::decay_t<decltype(out)>;
         const int LS = row_pitch(s.N, s.radices.empty() ? 1 : s.radices[0], rb, sizeof(E));
         const size_t sm = row_smem(s, rb, LS, sizeof(E), Out::staged);
-        allow_smem(k_fft_rows<A, Out>, sm);
-        k_fft_rows<A, Out><<<dim3((unsigned)cdiv(s.N, rb), npairs), RowNT<A>::value, sm, st>>>(
-            G, P, rb, magic(rb), LS, s.d_Rm, W, tw, out);
+        const auto kern = low ? k_fft_rows<A, Out, LOW_RADIX> : k_fft_rows<A, Out, MAX_RADIX>;
+        allow_smem(kern, sm);
+        kern<<<dim3((unsigned)cdiv(s.N, rb), npairs), RowNT<A>::value, sm, st>>>(G, P, rb, magic(rb), LS, s.d_Rm, W, tw, out);
     };
     auto rows = [&](int rb) {
         if constexpr (std::is_same<A, ArithF32>::value) {
@@ -973,8 +992,8 @@ abs_status run_fft_as(abs_ctx *ctx, const Setup &s, const Src &src, float *d_fie
 // Xt(., -t)) / 2i are Hermitian on the ring and Z = H1 + i H2.  The row pass therefore
 // gives the real fields F1 = FFT(H1) and F2 = FFT(H2) of the pair in its slots 2p and
 // 2p + 1, and the transforms of Xt(., +-t) are F1 +- i F2.  Same W layout as k_fft_cols.
-template <class A>
-__global__ void __launch_bounds__(FFT_NT) k_fft_cols_delay(RingGeom G, const __grid_constant__ FftPlan P, int CB,
+template <class A, int MAXR>
+__global__ void __launch_bounds__(FFT_NT, fft_min_blocks<A, MAXR>()) k_fft_cols_delay(RingGeom G, const __grid_constant__ FftPlan P, int CB,
                                                         const int64_t *__restrict__ q, const int32_t *__restrict__ Rm,
                                                         int t1, int Rr, const float4 *__restrict__ Xt,
                                                         const float4 *__restrict__ tw, typename A::E *__restrict__ W) {
@@ -998,7 +1017,7 @@ __global__ void __launch_bounds__(FFT_NT) k_fft_cols_delay(RingGeom G, const __g
         if (r2 < q0 || r2 >= q1) continue;
         l0[(size_t)c * G.N + (y < 0 ? y + G.N : y)] = A::from_cell(src[(size_t)(y + Rr) * side + (x + Rr)]);
     }
-    E *res = fft_lines<A>(l0, l1, CB, P, tw);
+    E *res = fft_lines<A, MAXR>(l0, l1, CB, P, tw);
     for (int e = threadIdx.x; e < CB * G.N; e += blockDim.x) {
         const int c = e / G.N, x = x0 + c;
         if (x < -Rp || x > Rp) continue;
@@ -1029,15 +1048,17 @@ abs_status run_fft_delay(abs_ctx *ctx, const Setup &s, int t_max, const float4 *
     const float4 *tw = A::table(s.d_tw, s.N);
     {
         StageTimer timer(ctx, "fft_cols_delay");
-        allow_smem(k_fft_cols_delay<A>, csm);
-        k_fft_cols_delay<A><<<dim3((unsigned)cdiv(2 * s.R + 1, CB), npairs), FFT_NT, csm, st>>>(
-            G, P, CB, s.d_q, s.d_Rm, t1, s.R, d_xt, tw, W);
+        const auto kern = low_radix(s) ? k_fft_cols_delay<A, LOW_RADIX> : k_fft_cols_delay<A, MAX_RADIX>;
+        allow_smem(kern, csm);
+        kern<<<dim3((unsigned)cdiv(2 * s.R + 1, CB), npairs), FFT_NT, csm, st>>>(G, P, CB, s.d_q, s.d_Rm, t1, s.R, d_xt, tw,
+                                                                                W);
     }
     {
         StageTimer timer(ctx, "fft_rows_delay");
-        allow_smem(k_fft_rows<A, FieldsOut>, rsm);
-        k_fft_rows<A, FieldsOut><<<dim3((unsigned)cdiv(s.N, RB), npairs), RowNT<A>::value, rsm, st>>>(
-            G, P, RB, magic(RB), LS, d_rm2, W, tw, FieldsOut{d_F});
+        const auto kern = low_radix(s) ? k_fft_rows<A, FieldsOut, LOW_RADIX> : k_fft_rows<A, FieldsOut, MAX_RADIX>;
+        allow_smem(kern, rsm);
+        kern<<<dim3((unsigned)cdiv(s.N, RB), npairs), RowNT<A>::value, rsm, st>>>(G, P, RB, magic(RB), LS, d_rm2, W, tw,
+                                                                                 FieldsOut{d_F});
     }
     return check_launch(ctx, "delay transforms");
 }
