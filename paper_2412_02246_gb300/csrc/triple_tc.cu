@@ -736,33 +736,49 @@ __global__ void __launch_bounds__(256) k_split_pad(int nb, int nbp, int64_t P, i
     f32[row + ((((u >> 2) ^ key) << 2) | (u & 3))] = 0.f;
 }
 
-// dense[x] = sum over pixel ranges of partial[r][x] (a fixed order).
-__global__ void __launch_bounds__(256) k_tc_reduce(int64_t dense, int n_ranges, const float *__restrict__ partial,
-                                                   double *__restrict__ out) {
-    const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= dense) return;
-    // eight loads in flight, added in range order into a double-float sum (TwoSum, then
-    // Fast2Sum; about 2^-44 relative, in FP32 arithmetic: GB300's FP64 pipe, which also
-    // converts, is narrow), widened to FP64 once
-    float sh = 0.f, sl = 0.f;
-    auto add = [&](float v) {
-        const float t = __fadd_rn(sh, v);
-        const float bp = __fsub_rn(t, sh);
-        const float e = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bp)), __fsub_rn(v, bp));
-        const float lo = __fadd_rn(sl, e);
-        sh = __fadd_rn(t, lo);
-        sl = __fsub_rn(lo, __fsub_rn(sh, t));
-    };
-    int r = 0;
-    for (; r + 8 <= n_ranges; r += 8) {
-        float v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = __ldcs(&partial[(size_t)(r + u) * dense + x]);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) add(v[u]);
+// dense[x] = sum over pixel ranges of partial[r][x] in double-float (TwoSum, then Fast2Sum; about
+// 2^-44 relative, in FP32 arithmetic: GB300's FP64 pipe, which also converts, is narrow), widened to
+// FP64 once: blockDim.y threads an entry take every blockDim.y-th range, eight loads in flight each,
+// and their sums are added in a fixed order.  Bound by memory with many entries, by the latency of a
+// thread's loads with few (a small grid's list has some 1e4 entries and 300 ranges: 29 us with one
+// thread an entry), hence the threads an entry gets (see tc_run).
+constexpr int RED_X = 64;
+struct DfSum {
+    float h = 0.f, l = 0.f;
+    __device__ __forceinline__ void add(float v, float vl = 0.f) {
+        const float t = __fadd_rn(h, v);
+        const float bp = __fsub_rn(t, h);
+        const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(t, bp)), __fsub_rn(v, bp));
+        const float lo = __fadd_rn(__fadd_rn(l, vl), e);
+        h = __fadd_rn(t, lo);
+        l = __fsub_rn(lo, __fsub_rn(h, t));
     }
-    for (; r < n_ranges; ++r) add(__ldcs(&partial[(size_t)r * dense + x]));
-    out[x] = (double)sh + (double)sl;
+};
+__global__ void __launch_bounds__(1024) k_tc_reduce(int64_t dense, int n_ranges, const float *__restrict__ partial,
+                                                    double *__restrict__ out) {
+    __shared__ float2 part[1024];
+    const int64_t x = (int64_t)blockIdx.x * RED_X + threadIdx.x;
+    const int step = blockDim.y;
+    DfSum s;
+    if (x < dense) {
+        int r = threadIdx.y;
+        for (; r + 7 * step < n_ranges; r += 8 * step) {
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = __ldcs(&partial[(size_t)(r + u * step) * dense + x]);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) s.add(v[u]);
+        }
+        for (; r < n_ranges; r += step) s.add(__ldcs(&partial[(size_t)r * dense + x]));
+    }
+    part[threadIdx.y * RED_X + threadIdx.x] = make_float2(s.h, s.l);
+    __syncthreads();
+    if (threadIdx.y || x >= dense) return;
+    for (int y = 1; y < step; ++y) {
+        const float2 p = part[y * RED_X + threadIdx.x];
+        s.add(p.x, p.y);
+    }
+    out[x] = (double)s.h + (double)s.l;
 }
 
 // S[t] = inv_p dense[pos[t]].
@@ -1023,7 +1039,10 @@ static abs_status tc_run(abs_ctx *ctx, const Setup &s, const TcPlanDev &pd, cons
     }
     {
         StageTimer timer(ctx, e0 ? nullptr : "tc_reduce");
-        k_tc_reduce<<<(int)cdiv(G.dense, 256), 256, 0, st>>>(G.dense, (int)ranges, partial, dsum);
+        // threads an entry: one while the entries alone fill the GPU, up to 16 below
+        int per = 1;
+        while (per < 16 && G.dense * per < (int64_t)ctx->sm_count * 2048 && per * 8 < ranges) per *= 2;
+        k_tc_reduce<<<(int)cdiv(G.dense, RED_X), dim3(RED_X, per), 0, st>>>(G.dense, (int)ranges, partial, dsum);
         k_tc_gather<<<(int)cdiv(n_trip, 256), 256, 0, st>>>(n_trip, 1.0 / (double)s.P, pd.d_pos,
                                                              dsum, d_sum);
     }
