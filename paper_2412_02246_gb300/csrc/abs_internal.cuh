@@ -52,6 +52,7 @@ struct Setup {
     size_t rg_at[7] = {0, 0, 0, 0, 0, 0, 0};
     int n_orb = 0;
     int item_cap[2] = {0, 0};
+    bool small_items = false;     // they are large enough for the shorter items
     // ordered closed-triangle counts of the full annuli [nb][nb][nb] (halved),
     // a property of the ring geometry, computed on first use
     unsigned long long *d_full_counts = nullptr;

@@ -71,7 +71,9 @@ namespace {
 constexpr int G1 = ABS_COUNT_G1;   // g1 cells per thread
 constexpr int KU = ABS_COUNT_KU;   // inner cells whose map loads are issued together
 constexpr int CT = 256;          // threads per counting CTA (max)
-constexpr int INNER = 512;       // inner cells per work item (bounds the work of one item)
+// inner cells per work item: INNER where that gives every CTA a few items, INNER_S where it would not
+// (an item of 1,024 x 512 visits takes 25 us, as long as a whole small grid should)
+constexpr int INNER = 512, INNER_S = 128;
 constexpr int GATHER_FUSED = 2048;   // longest triplet list gathered by the pair kernel's last CTA
 constexpr unsigned FULL = 0xffffffffu;
 
@@ -99,7 +101,8 @@ struct RingTables {
     uint8_t *nf;                 // [nO] filled upper-half cells of every orbit
     int32_t *cnt;                // [3][nb]: F, H (upper half), HO
     unsigned long long *fix;     // [nb][nb]: holes (upper half) of ring a with h / 2 in ring b
-    int *ctl;                    // [0], [1] items of list 0, 1; [2], [3] next item; [4] the route
+    int *ctl;                    // [0], [1] items of list 0, 1; [2], [3] next item; [4] the route;
+                                 // [5] inner cells of an item
 };
 
 __device__ __forceinline__ int64_t cell_index(int n, int gx, int gy) {
@@ -241,6 +244,8 @@ __device__ __forceinline__ int suffix_start(const CountGeom &G, int a, int b) {
 
 struct ItemArgs {
     int chunk, need_full, cap0, cap1;
+    int ctas;                                        // of the pair kernel
+    int small_ok;                                    // the lists hold items of INNER_S
     int4 *items0, *items1;
     int32_t *err;
     unsigned long long *tab0, *tabP, *tabM, *full;   // [nb^3]; full cleared when need_full
@@ -281,7 +286,7 @@ __global__ void __launch_bounds__(256) k_ring_finish(CountGeom G, float du, Ring
     if (!ia.items0) return;
     // the route: pairs visited by either (suffix sums over the rings b >= a)
     __shared__ int cF[ABS_MAX_BINS], cH[ABS_MAX_BINS];
-    __shared__ int use_holes_s;
+    __shared__ int use_holes_s, inner_s;
     for (int i = threadIdx.x; i < nb; i += 256) {
         cF[i] = T.cnt[i];
         cH[i] = T.cnt[nb + i];
@@ -317,11 +322,18 @@ __global__ void __launch_bounds__(256) k_ring_finish(CountGeom G, float du, Ring
             dir += __shfl_xor_sync(FULL, dir, o);
             hol += __shfl_xor_sync(FULL, hol, o);
         }
-        if (lane == 0) use_holes_s = hol < dir ? 1 : 0;
+        if (lane == 0) {
+            use_holes_s = hol < dir ? 1 : 0;
+            const unsigned long long visits = ia.need_full ? ~0ull : hol < dir ? hol : dir;
+            inner_s = ia.small_ok && visits / ((unsigned long long)ia.chunk * INNER) < 4ull * ia.ctas ? INNER_S : INNER;
+        }
     }
     __syncthreads();
-    const int holes = use_holes_s;
-    if (blockIdx.x == 0 && threadIdx.x == 0) T.ctl[4] = holes;
+    const int holes = use_holes_s, inner = inner_s;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        T.ctl[4] = holes;
+        T.ctl[5] = inner;
+    }
     // the tables' rows that will be added to (the holes' route: rings a with holes only)
     const int64_t row = (int64_t)nb * nb;
     for (int a = blockIdx.x; a < nb; a += gridDim.x) {
@@ -359,7 +371,7 @@ __global__ void __launch_bounds__(256) k_ring_finish(CountGeom G, float du, Ring
         }
         const bool outer_x = nx >= ny;
         const int no = outer_x ? nx : ny, ni = outer_x ? ny : nx;
-        const int n_ic = (ni + INNER - 1) / INNER;
+        const int n_ic = (ni + inner - 1) / inner;
         const int cnt = ni > 0 ? (no + ia.chunk - 1) / ia.chunk * n_ic : 0;
         const int lst = job >= JOB_P ? 1 : 0;
         // places: an inclusive scan over the warp, one reservation a list
@@ -394,7 +406,7 @@ __global__ void __launch_bounds__(256) k_ring_finish(CountGeom G, float du, Ring
             }
             const int4 P = w_pair[warp][lo];
             const int c = t - w_pos[warp][lo], oc = c / P.y, ic = c - oc * P.y;
-            const int4 item = make_int4(P.x, oc * ia.chunk, ic * INNER, P.z);
+            const int4 item = make_int4(P.x, oc * ia.chunk, ic * inner, P.z);
             if (((P.x >> 16) & 7) >= JOB_P) {
                 if (base1 + t - t0 < ia.cap1) ia.items1[base1 + t - t0] = item;
             } else if (base0 + t < ia.cap0) {
@@ -507,6 +519,7 @@ __global__ void __launch_bounds__(CT) k_count_pairs(CountGeom G, RingTables T, c
     uint16_t *myhist = hist + (size_t)warp * hs * 32 + lane;
     const uint32_t span = 2u * (uint32_t)G.R;   // |x1 + x2| <= R  <=>  x1 + R + x2 in [0, 2R]
     __shared__ int it_s;
+    const int inner = T.ctl[5];
     bool clean = false;
     for (int lst = 0; lst < 2; ++lst) {
         const int ni = min(T.ctl[lst], lst ? cap1 : cap0);
@@ -557,7 +570,7 @@ __global__ void __launch_bounds__(CT) k_count_pairs(CountGeom G, RingTables T, c
                 return make_int4(neg ? -l : l, neg ? -g.x : g.x, job == JOB_M ? 2 * (g.y * G.K + g.x) : 1, 1);
             };
             const int no = outer_x ? nx : ny;
-            const int nin = min(INNER, (outer_x ? ny : nx) - I.z);
+            const int nin = min(inner, (outer_x ? ny : nx) - I.z);
             int lin1[G1], xr1[G1], k1[G1];   // lin, x + R and half-plane key of this thread's outer cells
             uint32_t w1[G1];
 #pragma unroll
@@ -670,17 +683,25 @@ bool make_ring_geometry(Setup &s) {
     s.n_orb = (int)orb.size();
     // work items at most: DIRECT or Q in list 0; P, M and FULL in list 1 (every list at its longest)
     const int64_t chunk = (int64_t)std::max(count_warps(nb), 1) * 32 * G1;
-    auto items = [&](int64_t x, int64_t y) { return cdiv(std::max(x, y), chunk) * cdiv(std::min(x, y), INNER); };
     int64_t c0 = 0, c1 = 0;
-    for (int a = 0; a < nb; ++a)
-        for (int b = 0; b < nb; ++b) {
-            const int64_t ua = up_off[a + 1] - up_off[a], ub = up_off[b + 1] - up_off[b], oa = orb_off[a + 1] - orb_off[a];
-            if (a <= b) {
-                c0 += items(ua, 2 * ub);
-                c1 += items(ua, 2 * ub) + items(oa, 2 * ub);
+    for (int inner : {INNER, INNER_S}) {
+        auto items = [&](int64_t x, int64_t y) { return cdiv(std::max(x, y), chunk) * cdiv(std::min(x, y), inner); };
+        int64_t n0 = 0, n1 = 0;
+        for (int a = 0; a < nb; ++a)
+            for (int b = 0; b < nb; ++b) {
+                const int64_t ua = up_off[a + 1] - up_off[a], ub = up_off[b + 1] - up_off[b], oa = orb_off[a + 1] - orb_off[a];
+                if (a <= b) {
+                    n0 += items(ua, 2 * ub);
+                    n1 += items(ua, 2 * ub) + items(oa, 2 * ub);
+                }
+                n1 += items(oa, ub);
             }
-            c1 += items(oa, ub);
+        s.small_items = inner == INNER_S && std::max(n0, n1) <= 1 << 21;   // 32 MB a list at most
+        if (inner == INNER || s.small_items) {
+            c0 = n0;
+            c1 = n1;
         }
+    }
     s.item_cap[0] = (int)std::min<int64_t>(std::max<int64_t>(c0, 1), 1 << 26);
     s.item_cap[1] = (int)std::min<int64_t>(std::max<int64_t>(c1, 1), 1 << 26);
     const void *src[7] = {up.data(), up_ring.data(), up_off.data(), orb.data(), orb_ring.data(), orb_off.data(), map.data()};
@@ -778,7 +799,8 @@ abs_status launch_counts(abs_ctx *ctx, const Setup &s, const uint8_t *d_mask, in
     }
     if (!items0 || !items1 || !ticket || !tabs || !ms.d_full_counts) return fail(ctx, ABS_ERR_OOM, "count workspace");
     unsigned long long *tab0 = tabs, *tabP = tabs + tn, *tabM = tabs + 2 * tn, *full = ms.d_full_counts;
-    ItemArgs ia{threads * G1, ms.full_counts_ready ? 0 : 1, cap0, cap1, items0, items1, ctx->d_err, tab0, tabP, tabM, full};
+    ItemArgs ia{threads * G1, ms.full_counts_ready ? 0 : 1, cap0, cap1, ctx->sm_count * per_sm, s.small_items ? 1 : 0,
+                items0, items1, ctx->d_err, tab0, tabP, tabM, full};
     ABS_CHECK(ring_tables(ctx, s, d_mask, d_accw, T, d_ellbar, &ia));
     {
         // long lists are gathered by a launch of their own (one CTA takes 0.3 ms for 1e5 triplets), short
