@@ -725,6 +725,21 @@ abs_status abs_triple(abs_ctx *ctx, const abs_config *cfg, const float *d_fields
     if (d_sum && !d_fields) return fail(ctx, ABS_ERR_INVALID_ARG, "d_fields is NULL");
     if (d_count && !d_mask) return fail(ctx, ABS_ERR_INVALID_ARG, "d_mask is NULL");
     ABS_CHECK(launch_check_triplets(ctx, *s, n_trip, d_ijk));
+    // the sums and the counts share nothing: the counts run on the side stream beside the sums (not while
+    // profiling stages)
+    const bool fork = d_sum && d_count && ctx->side && !ctx->profiling;
+    if (fork) {
+        cudaEventRecord(ctx->ev_fork, ctx->stream);
+        cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0);
+        cudaStream_t main = ctx->stream;
+        ctx->stream = ctx->side;
+        const abs_status sc = launch_counts(ctx, *s, d_mask, n_trip, d_ijk, d_count, nullptr);
+        cudaEventRecord(ctx->ev_join, ctx->side);
+        ctx->stream = main;
+        const abs_status ss = launch_triple_sums(ctx, *s, d_fields, n_trip, d_ijk, d_sum);
+        cudaStreamWaitEvent(ctx->stream, ctx->ev_join, 0);
+        return ss != ABS_OK ? ss : sc;
+    }
     if (d_sum) ABS_CHECK(launch_triple_sums(ctx, *s, d_fields, n_trip, d_ijk, d_sum));
     if (d_count) ABS_CHECK(launch_counts(ctx, *s, d_mask, n_trip, d_ijk, d_count, nullptr));
     return ABS_OK;

@@ -74,7 +74,7 @@ constexpr int CT = 256;          // threads per counting CTA (max)
 // inner cells per work item: INNER where that gives every CTA a few items, INNER_S where it would not
 // (an item of 1,024 x 512 visits takes 25 us, as long as a whole small grid should)
 constexpr int INNER = 512, INNER_S = 128;
-constexpr int GATHER_FUSED = 2048;   // longest triplet list gathered by the pair kernel's last CTA
+constexpr int GATHER_FUSED = CT;     // longest triplet list gathered by the pair kernel's last CTA
 constexpr unsigned FULL = 0xffffffffu;
 
 struct CountGeom {
@@ -519,6 +519,7 @@ __global__ void __launch_bounds__(CT) k_count_pairs(CountGeom G, RingTables T, c
     uint16_t *myhist = hist + (size_t)warp * hs * 32 + lane;
     const uint32_t span = 2u * (uint32_t)G.R;   // |x1 + x2| <= R  <=>  x1 + R + x2 in [0, 2R]
     __shared__ int it_s;
+    __shared__ int4 item_s;
     const int inner = T.ctl[5];
     bool clean = false;
     for (int lst = 0; lst < 2; ++lst) {
@@ -527,12 +528,21 @@ __global__ void __launch_bounds__(CT) k_count_pairs(CountGeom G, RingTables T, c
         const uint8_t *map_g = lst ? G.mapA : T.mapF, *map = MAP_IN_SMEM ? map_s : map_g;
         const int4 *items = lst ? items1 : items0;
         bool loaded = !MAP_IN_SMEM;
+        // thread 0 fetches the next item while the CTA counts this one (dynamic: items differ in size)
+        int next = 0;
+        int4 nitem = make_int4(0, 0, 0, 0);
+        if (threadIdx.x == 0) {
+            next = atomicAdd(T.ctl + 2 + lst, 1);
+            if (next < ni) nitem = items[next];
+        }
         for (;;) {
+            if (threadIdx.x == 0) {
+                it_s = next;
+                item_s = nitem;
+            }
             __syncthreads();
-            if (threadIdx.x == 0) it_s = atomicAdd(T.ctl + 2 + lst, 1);   // dynamic: items differ in size
-            __syncthreads();
-            const int it = it_s;
-            if (it >= ni) break;
+            if (it_s >= ni) break;
+            const int4 I = item_s;
             if (!loaded) {   // a CTA that takes no item loads no map and clears nothing
                 const int64_t mb = G.base + 1, nv = mb / 16;
                 for (int64_t i = threadIdx.x; i < nv; i += blockDim.x) ((uint4 *)map_s)[i] = ((const uint4 *)map_g)[i];
@@ -543,7 +553,6 @@ __global__ void __launch_bounds__(CT) k_count_pairs(CountGeom G, RingTables T, c
                 for (int i = threadIdx.x; i < hwords; i += blockDim.x) hist32[i] = 0u;
                 clean = true;
             }
-            const int4 I = items[it];
             const int a = I.x & 255, b = (I.x >> 8) & 255, job = (I.x >> 16) & 7;
             const bool outer_x = (I.x & (1 << 24)) != 0;
             const bool orbit = job >= JOB_M;       // X holds packed orbits
@@ -587,8 +596,10 @@ __global__ void __launch_bounds__(CT) k_count_pairs(CountGeom G, RingTables T, c
             }
             for (int k = threadIdx.x; k < nin; k += blockDim.x) stage[k] = outer_x ? load_y(I.z + k) : load_x(I.z + k);
             __syncthreads();
+            if (threadIdx.x == 0) next = atomicAdd(T.ctl + 2 + lst, 1);
             if (orbit) count_inner<true>(stage, nin, map, lin1, xr1, k1, w1, span, myhist);
             else count_inner<false>(stage, nin, map, lin1, xr1, k1, w1, span, myhist);
+            if (threadIdx.x == 0 && next < ni) nitem = items[next];
             __syncthreads();
             unsigned long long *tab = job == JOB_P ? tabP : job == JOB_M ? tabM : job == JOB_FULL ? full : tab0;
             for (int k = 1 + warp; k < hs; k += nwarps) {
@@ -602,6 +613,7 @@ __global__ void __launch_bounds__(CT) k_count_pairs(CountGeom G, RingTables T, c
             __syncthreads();
             for (int k = threadIdx.x; k < hwords; k += blockDim.x) hist32[k] = 0u;
         }
+        __syncthreads();   // everyone has seen the end of the list
     }
     if (!ga.ticket) return;
     __shared__ bool last;
