@@ -53,6 +53,9 @@ struct Setup {
     int n_orb = 0;
     int item_cap[2] = {0, 0};
     bool small_items = false;     // they are large enough for the shorter items
+    // realisations of this configuration have been through lanes 0 .. lanes_ready - 1 (their workspaces
+    // exist) with lists of lanes_trip triplets
+    mutable int32_t lanes_ready = 0, lanes_trip = 0;
     // ordered closed-triangle counts of the full annuli [nb][nb][nb] (halved),
     // a property of the ring geometry, computed on first use
     unsigned long long *d_full_counts = nullptr;
@@ -148,6 +151,8 @@ namespace absk {
 
 // Concurrent lanes of abs_estimate_batched (items round-robin over them).
 constexpr int ABS_BATCH_LANES = 4;
+// Largest realisation (accumulators and fields, bytes) that estimates of several run on lanes.
+constexpr size_t LANE_REAL_BYTES = (size_t)512 << 20;
 // Creates lanes of ctx (child contexts with their own streams and workspaces, sharing its
 // device error word) until it has K.
 abs_status ensure_lanes(abs_ctx *ctx, int K);
@@ -180,9 +185,11 @@ abs_status launch_grid_plan(abs_ctx *ctx, const Setup &s, int64_t n_vis, const f
                             bool rings_only = false);
 // With d_grid == d_wsum == nullptr only the FP64 accumulators are produced.
 // acc_zeroed: the caller has already cleared
-// the accumulators (grid_acc_buffers) on this stream's timeline.
+// the accumulators (grid_acc_buffers) on this stream's timeline.  plan: the context
+// whose plan it reads (nullptr: its own).
 abs_status launch_grid_accumulate(abs_ctx *ctx, const Setup &s, int64_t n_vis, const float *d_vis,
-                                  float *d_grid, float *d_wsum, uint8_t *d_mask, bool acc_zeroed = false);
+                                  float *d_grid, float *d_wsum, uint8_t *d_mask, bool acc_zeroed = false,
+                                  abs_ctx *plan = nullptr);
 abs_status launch_filter_fft(abs_ctx *ctx, const Setup &s, const float *d_grid,
                              const float *d_wsum, const uint8_t *d_mask, float *d_fields);
 // The split-BF16 kernel's operands: the fields as three chunk-blocked planes

@@ -759,13 +759,13 @@ void grid_acc_buffers(abs_ctx *ctx, const Setup &s, double **acc) {
 }
 
 abs_status launch_grid_accumulate(abs_ctx *ctx, const Setup &s, int64_t n_vis, const float *d_vis,
-                                  float *d_grid, float *d_wsum, uint8_t *d_mask, bool acc_zeroed) {
+                                  float *d_grid, float *d_wsum, uint8_t *d_mask, bool acc_zeroed, abs_ctx *plan) {
     // the estimate path (no FP32 outputs; its plan was made with rings_only) accumulates what
     // its weighting needs
     const bool estimate = !d_grid && !d_wsum;
     const GridGeom G = geom(s, estimate);
     PlanBufs b;
-    if (!plan_bufs(ctx, G, n_vis, b)) return fail(ctx, ABS_ERR_OOM, "grid plan workspace");
+    if (!plan_bufs(plan ? plan : ctx, G, n_vis, b)) return fail(ctx, ABS_ERR_OOM, "grid plan workspace");
     const int64_t cells = (int64_t)s.n * s.n;
     const int wm = !estimate ? GW_SUM
                    : s.weight_mode == ABS_W_PAPER_LITERAL ? GW_COUNT
