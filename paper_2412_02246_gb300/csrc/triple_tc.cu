@@ -98,11 +98,13 @@ constexpr int FPX = KC / FQ;            // pixels of a chunk per forming thread
 // thread issues at most one tcgen05.mma every ~45 cycles, so the tiles of a set issue in parallel.
 constexpr int NISS = ABS_TC_ISSUERS;
 constexpr int FW0 = 1 + NISS;           // first forming warp (warp 0 loads, warps 1 .. NISS issue)
-constexpr int NT = (NFORM + FW0) * 32;  // threads per CTA
+constexpr int DW0 = FW0 + NFORM;        // first draining warp
+constexpr int NDRAIN = 8;               // draining warps, two a tensor-memory lane quadrant
+constexpr int NT = (DW0 + NDRAIN) * 32; // threads per CTA
 // registers per thread: the register file is split over the SM's four schedulers (16,384
 // each) and warps are dealt to them in turn, so the scheduler with the most warps
-// (3 of 10 or 11, or 5 of 18 or 19) bounds it, in steps of 8
-#define TC_MAXREG (ABS_TC_FORMERS == 8 ? 168 : 96)
+// (5 of 19) bounds it, in steps of 8
+#define TC_MAXREG 96
 #ifndef ABS_TC_ASLOTS
 #define ABS_TC_ASLOTS 2
 #endif
@@ -127,8 +129,9 @@ constexpr int DRAIN = ABS_TC_DRAIN;  // chunks accumulated in tensor memory befo
 constexpr int MAX_SET_COLS = ABS_TC_SET_COLS;
 static_assert(NABUF * A_COLS + 2 * MAX_SET_COLS <= TMEM_COLS, "A buffers and two regions fit tensor memory");
 constexpr int MAX_TILE_N = 128;      // MMA N of a tile (wider column ranges are cut into several tiles)
-constexpr int MAXBLK = (MAX_SET_COLS / 8 + FQ - 1) / FQ;     // drain blocks of 8 columns per forming thread
-constexpr int MAXSLOT = 8 * MAXBLK;  // long accumulators per forming thread
+constexpr int DQ = NDRAIN / 4;       // draining warps per quadrant
+constexpr int MAXBLK = (MAX_SET_COLS / 8 + DQ - 1) / DQ;     // drain blocks of 8 columns per draining thread
+constexpr int MAXSLOT = 8 * MAXBLK;  // long accumulators per draining thread
 // A wait suspends the warp for up to WAIT_HINT_NS per try (it resumes as soon as the
 // phase completes, so waiting warps take no issue slots), at most WAIT_LIMIT tries.
 constexpr uint32_t WAIT_HINT_NS = 100000;
@@ -346,8 +349,8 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
     __shared__ int t_ilo[MAX_TILES], t_n[MAX_TILES], t_col[MAX_TILES], sum_n;
     __shared__ int64_t t_off[MAX_TILES];
     __shared__ short2 rows_s[MAX_TILES][TM];
-    __shared__ int blk_col[FQ][MAXBLK], n_blk[FQ];   // drain blocks of 8 columns per forming warp of a quadrant
-    __shared__ int64_t blk_out[FQ][MAXBLK];
+    __shared__ int blk_col[DQ][MAXBLK], n_blk[DQ];   // drain blocks of 8 columns per draining warp of a quadrant
+    __shared__ int64_t blk_out[DQ][MAXBLK];
     // stages on a 1024-byte boundary (the 128-byte swizzle's atom); the launch adds 1 KB of slack
     uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     const int warp = uni((int)(threadIdx.x >> 5)), lane = threadIdx.x & 31;
@@ -360,7 +363,7 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
         for (int b = 0; b < ASLOTS * MAX_TILES; ++b) mbar_init(smem_u32(&a_full[b]), NFORM);
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&d_full[b]), NISS);
-            mbar_init(smem_u32(&d_empty[b]), NFORM);
+            mbar_init(smem_u32(&d_empty[b]), NDRAIN);
         }
         mbar_init(smem_u32(&fin), NISS);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -383,9 +386,6 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
     for (int x = 0; x < ASLOTS; ++x) hst[x] = hsu[x] = 0;
     int grp = 0;             // accumulation groups so far (region grp & 1, its use grp >> 1)
     int issued = 0;          // stages the loader filled (for the drain)
-    float accl[MAXSLOT];     // formers: this thread's long accumulators (FP32, rounded to nearest)
-#pragma unroll
-    for (int x = 0; x < MAXSLOT; ++x) accl[x] = 0.f;
     for (;;) {
         // every thread is between items here, and no role writes the abort flag; the next
         // item comes from the launch's work counter (items in pixel-range order, so the
@@ -415,11 +415,11 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
         if (threadIdx.x == 0) {
             // tile columns inside an accumulation region; drain blocks dealt round robin
             int col = 0, b = 0;
-            for (int h = 0; h < FQ; ++h) n_blk[h] = 0;
+            for (int h = 0; h < DQ; ++h) n_blk[h] = 0;
             for (int t = 0; t < S.ntiles; ++t) {
                 t_col[t] = col;
                 for (int c0 = 0; c0 < t_n[t]; c0 += 8, ++b) {
-                    const int h = b % FQ, k = n_blk[h]++;
+                    const int h = b % DQ, k = n_blk[h]++;
                     blk_col[h][k] = col + c0;
                     blk_out[h][k] = t_off[t] + (int64_t)c0 * TM;
                 }
@@ -528,13 +528,12 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
                 }
                 if (++gc == DRAIN) gc = 0;
             }
-        } else {
-            // ---------------- formers; after the first chunk of each group they drain the group before
+        } else if (warp < DW0) {
+            // ---------------- formers
             const int q = warp & 3;                   // tensor-memory lanes 32 q .. 32 q + 31
-            const int h = (warp - FW0) >> 2;          // pixel part of the chunk (FPX pixels), drain blocks
+            const int h = (warp - FW0) >> 2;          // pixel part of the chunk (FPX pixels)
             const int row = 32 * q + lane;
             const uint32_t lane_base = tmem + ((uint32_t)(32 * q) << 16);
-            const int nb_h = n_blk[h];
             // this thread's rows of the set's tiles: offsets of D_j and D_k in an F window (a row the tile
             // does not have forms the window's first ring; its sums are never read)
             uint32_t rel_j[MAX_TILES], rel_k[MAX_TILES];
@@ -544,103 +543,104 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
                 rel_j[t] = jk.x >= 0 ? frow_rel(jk.x, S.f_lo, (h * FPX) / 4) : 0u;
                 rel_k[t] = jk.x >= 0 ? frow_rel(jk.y, S.f_lo, (h * FPX) / 4) : 0u;
             }
-            int gdrained = grp;                       // this item's first group
             bool fail_f = false;
             // a barrier test takes over 100 cycles to answer, so the next chunk's two are asked for before the
             // end of this one: the copies have landed; the MMAs that read the next chunk's A slot are done
             bool full_ok = false, done_ok = false;
-            // chunk c is formed; after the first chunk of a group (and after the last chunk) the group
-            // before is drained: its accumulation region is added into accl and released
-            for (int c = 0; c <= nchunks && !fail_f; ++c) {
-                if (c < nchunks) {
-                    if (!full_ok && !mbar_wait(smem_u32(&full[st]), (uint32_t)(su & 1), &abort_s)) {
-                        fail_f = true;
-                        break;
-                    }
-                    // the F window
-                    const uint8_t *F = smem + (size_t)st * G.stage_bytes + 2 * b_bytes;
-                    // the A buffers of this chunk's pair were read by the MMAs of chunk cg - 2
-                    if (!done_ok && cg >= ASLOTS &&
-                        !mbar_wait(smem_u32(&done[hst[0]]), (uint32_t)(hsu[0] & 1), &abort_s)) {
-                        fail_f = true;
-                        break;
-                    }
-#pragma unroll
-                    for (int x = 0; x + 1 < ASLOTS; ++x) {
-                        hst[x] = hst[x + 1];
-                        hsu[x] = hsu[x + 1];
-                    }
-                    hst[ASLOTS - 1] = st;
-                    hsu[ASLOTS - 1] = su;
-                    const int nst = st + 1 == G.n_stages ? 0 : st + 1, nsu = st + 1 == G.n_stages ? su + 1 : su;
-                    const uint32_t Fs = after_wait(smem_u32(F));
-#pragma unroll
-                    for (int t = 0; t < MAX_TILES; ++t) {
-                        if (t >= S.ntiles) break;
-                        const uint32_t ta =
-                            lane_base + (uint32_t)(((cg & (ASLOTS - 1)) * MAX_TILES + t) * A_COLS + (FPX / 2) * h);
-                        const uint32_t pj = Fs + rel_j[t], pk = Fs + rel_k[t];
-                        // 16 pixels at a time: products, hi / lo split, 8 packed pairs of each to tensor memory
-#pragma unroll
-                        for (int part = 0; part < FPX / 16; ++part) {
-                            uint32_t hi[8], lo[8];
-#pragma unroll
-                            for (int cc = 0; cc < 4; ++cc) {
-                                const uint32_t w = (uint32_t)(4 * part + cc) << 4;
-                                const float4 x = lds128(pj ^ w), y = lds128(pk ^ w);
-                                split2(__fmul2_rn(make_float2(x.x, x.y), make_float2(y.x, y.y)), hi[2 * cc],
-                                       lo[2 * cc]);
-                                split2(__fmul2_rn(make_float2(x.z, x.w), make_float2(y.z, y.w)), hi[2 * cc + 1],
-                                       lo[2 * cc + 1]);
-                            }
-                            tmem_st(ta + 8u * part, hi);
-                            tmem_st(ta + 32u + 8u * part, lo);
-                        }
-                        if (t == S.ntiles - 1 && c + 1 < nchunks) {
-                            full_ok = mbar_test(smem_u32(&full[nst]), (uint32_t)(nsu & 1));
-                            done_ok = cg + 1 >= ASLOTS && mbar_test(smem_u32(&done[hst[0]]), (uint32_t)(hsu[0] & 1));
-                        }
-                        // tile t's A buffers are complete: its issuer may start while the next is formed
-                        asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
-                        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&a_full[(cg & (ASLOTS - 1)) * MAX_TILES + t]));
-                    }
-                    // tiles the set does not have: their barriers keep step with the chunks
-                    if (lane == 0)
-                        for (int t = S.ntiles; t < MAX_TILES; ++t)
-                            mbar_arrive(smem_u32(&a_full[(cg & (ASLOTS - 1)) * MAX_TILES + t]));
-                    ++cg;
-                    st = nst;
-                    su = nsu;
+            for (int c = 0; c < nchunks; ++c) {
+                if (!full_ok && !mbar_wait(smem_u32(&full[st]), (uint32_t)(su & 1), &abort_s)) {
+                    fail_f = true;
+                    break;
                 }
-                if (c == nchunks || (c % DRAIN == 0 && c > 0)) {
-                    const int g = gdrained;
-                    if (!mbar_wait(smem_u32(&d_full[g & 1]), (uint32_t)((g >> 1) & 1), &abort_s)) {
-                        fail_f = true;
-                        break;
+                // the F window
+                const uint8_t *F = smem + (size_t)st * G.stage_bytes + 2 * b_bytes;
+                // the A buffers of this chunk's pair were read by the MMAs of chunk cg - 2
+                if (!done_ok && cg >= ASLOTS &&
+                    !mbar_wait(smem_u32(&done[hst[0]]), (uint32_t)(hsu[0] & 1), &abort_s)) {
+                    fail_f = true;
+                    break;
+                }
+#pragma unroll
+                for (int x = 0; x + 1 < ASLOTS; ++x) {
+                    hst[x] = hst[x + 1];
+                    hsu[x] = hsu[x + 1];
+                }
+                hst[ASLOTS - 1] = st;
+                hsu[ASLOTS - 1] = su;
+                const int nst = st + 1 == G.n_stages ? 0 : st + 1, nsu = st + 1 == G.n_stages ? su + 1 : su;
+                const uint32_t Fs = after_wait(smem_u32(F));
+#pragma unroll
+                for (int t = 0; t < MAX_TILES; ++t) {
+                    if (t >= S.ntiles) break;
+                    const uint32_t ta =
+                        lane_base + (uint32_t)(((cg & (ASLOTS - 1)) * MAX_TILES + t) * A_COLS + (FPX / 2) * h);
+                    const uint32_t pj = Fs + rel_j[t], pk = Fs + rel_k[t];
+                    // 16 pixels at a time: products, hi / lo split, 8 packed pairs of each to tensor memory
+#pragma unroll
+                    for (int part = 0; part < FPX / 16; ++part) {
+                        uint32_t hi[8], lo[8];
+#pragma unroll
+                        for (int cc = 0; cc < 4; ++cc) {
+                            const uint32_t w = (uint32_t)(4 * part + cc) << 4;
+                            const float4 x = lds128(pj ^ w), y = lds128(pk ^ w);
+                            split2(__fmul2_rn(make_float2(x.x, x.y), make_float2(y.x, y.y)), hi[2 * cc],
+                                   lo[2 * cc]);
+                            split2(__fmul2_rn(make_float2(x.z, x.w), make_float2(y.z, y.w)), hi[2 * cc + 1],
+                                   lo[2 * cc + 1]);
+                        }
+                        tmem_st(ta + 8u * part, hi);
+                        tmem_st(ta + 32u + 8u * part, lo);
                     }
-                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    const uint32_t base = lane_base + (uint32_t)(NABUF * A_COLS + (g & 1) * region_cols);
-#pragma unroll
-                    for (int b0 = 0; b0 < MAXBLK; b0 += 4) {
-                        uint32_t v[4][8];
-#pragma unroll
-                        for (int b = 0; b < 4; ++b)
-                            if (b0 + b < MAXBLK && b0 + b < nb_h) tmem_ld8(base + (uint32_t)blk_col[h][b0 + b], v[b]);
-                        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-                        for (int b = 0; b < 4; ++b)
-                            if (b0 + b < MAXBLK && b0 + b < nb_h) {
-#pragma unroll
-                                for (int x = 0; x < 8; ++x) accl[8 * (b0 + b) + x] += __uint_as_float(v[b][x]);
-                            }
+                    if (t == S.ntiles - 1 && c + 1 < nchunks) {
+                        full_ok = mbar_test(smem_u32(&full[nst]), (uint32_t)(nsu & 1));
+                        done_ok = cg + 1 >= ASLOTS && mbar_test(smem_u32(&done[hst[0]]), (uint32_t)(hsu[0] & 1));
                     }
+                    // tile t's A buffers are complete: its issuer may start while the next is formed
+                    asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
                     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&d_empty[g & 1]));
-                    ++gdrained;
+                    if (lane == 0) mbar_arrive(smem_u32(&a_full[(cg & (ASLOTS - 1)) * MAX_TILES + t]));
                 }
+                // tiles the set does not have: their barriers keep step with the chunks
+                if (lane == 0)
+                    for (int t = S.ntiles; t < MAX_TILES; ++t)
+                        mbar_arrive(smem_u32(&a_full[(cg & (ASLOTS - 1)) * MAX_TILES + t]));
+                ++cg;
+                st = nst;
+                su = nsu;
+            }
+            if (fail_f) abort_s = 1;
+        } else {
+            // ---------------- drainers: every group's accumulation region is added into accl and released
+            const int q = warp & 3;
+            const int h = (warp - DW0) >> 2;          // drain blocks
+            const int row = 32 * q + lane;
+            const uint32_t lane_base = tmem + ((uint32_t)(32 * q) << 16);
+            const int nb_h = n_blk[h];
+            bool fail_f = false;
+            float accl[MAXSLOT];                      // this thread's long accumulators (FP32, rounded to nearest)
+#pragma unroll
+            for (int x = 0; x < MAXSLOT; ++x) accl[x] = 0.f;
+            for (int c = 0; c < nchunks; c += DRAIN) {
+                if (!mbar_wait(smem_u32(&d_full[grp & 1]), (uint32_t)((grp >> 1) & 1), &abort_s)) {
+                    fail_f = true;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                const uint32_t base = lane_base + (uint32_t)(NABUF * A_COLS + (grp & 1) * region_cols);
+#pragma unroll
+                for (int b = 0; b < MAXBLK; ++b) {   // one block at a time: the accumulators fill the registers
+                    if (b >= nb_h) break;
+                    uint32_t v[8];
+                    tmem_ld8(base + (uint32_t)blk_col[h][b], v);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+                    for (int x = 0; x < 8; ++x) accl[8 * b + x] += __uint_as_float(v[x]);
+                }
+                asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&d_empty[grp & 1]));
+                ++grp;
             }
             if (fail_f) {
                 abort_s = 1;
@@ -652,13 +652,9 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
                     if (b < nb_h) {
                         float *o = out + blk_out[h][b];
 #pragma unroll
-                        for (int x = 0; x < 8; ++x) {
-                            o[x * TM] = accl[8 * b + x];
-                            accl[8 * b + x] = 0.f;
-                        }
+                        for (int x = 0; x < 8; ++x) o[x * TM] = accl[8 * b + x];
                     }
             }
-            grp = gdrained;                           // formers keep their own count of groups
         }
     }
     // every role is done (or gave up): copies and MMAs in flight land before the memory goes
