@@ -558,7 +558,7 @@ __global__ void __launch_bounds__(FFT_NT, fft_min_blocks<A, MAXR>()) k_fft_cols(
 // along x.  The first Stockham pass reads its inputs straight from the column
 // pass's output (zero outside |x| <= R of the pair; consecutive threads take
 // consecutive rows of one column, which are adjacent there), the middle passes
-// go between two shared-memory line buffers (line pitch LS), and the last pass
+// go between two shared-memory line buffers (see RowShape), and the last pass
 // writes each output row of both fields to global memory, consecutive threads
 // consecutive pixels.  Rounding aside, the same transform as fft_lines.
 // Where the row pass puts the fields of a ring pair (a, b; b = -1 for none).
@@ -615,10 +615,10 @@ struct PlanesOut {
         *(float4 *)(o.f32 + row + (size_t)(((2 * unit) ^ key) << 2)) = make_float4(v[0], v[1], v[2], v[3]);
         *(float4 *)(o.f32 + row + (size_t)(((2 * unit + 1) ^ key) << 2)) = make_float4(v[4], v[5], v[6], v[7]);
     }
-    // The CTA's rows py0 .. py0 + rb - 1 (res: line r at r LS, complex (D_a, D_b)):
-    // the whole 8-pixel groups inside the block vectorised, the ragged ends one by one.
+    // The CTA's rows py0 .. py0 + rb - 1 (res: pixel n of line r at r LS + n + (n >> skew), complex
+    // (D_a, D_b)): the whole 8-pixel groups inside the block vectorised, the ragged ends one by one.
     template <class A>
-    __device__ void store_block(const RingGeom &G, int a, int b, const typename A::E *res, int LS, int py0,
+    __device__ void store_block(const RingGeom &G, int a, int b, const typename A::E *res, int LS, int skew, int py0,
                                 int rb) const {
         const size_t P0 = (size_t)py0 * G.N, P1 = P0 + (size_t)rb * G.N;
         const size_t g0 = (P0 + 7) / 8, g1 = P1 / 8;
@@ -629,7 +629,7 @@ struct PlanesOut {
             float va[8], vb[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-                const typename A::E v = res[(size_t)r * LS + n];
+                const typename A::E v = res[r * LS + n + (n >> skew)];
                 va[e] = A::re(v);
                 vb[e] = A::im(v);
                 if (++n == G.N) {
@@ -643,16 +643,32 @@ struct PlanesOut {
         // pixels of a group shared with the neighbouring block
         const size_t e0 = g0 * 8 > P1 ? P1 : g0 * 8, e1 = g1 * 8 < e0 ? e0 : g1 * 8;
         for (size_t pix = P0 + threadIdx.x; pix < e0; pix += blockDim.x) {
-            const int local = (int)(pix - P0), r = local / G.N;
-            const typename A::E v = res[(size_t)r * LS + (local - r * G.N)];
+            const int local = (int)(pix - P0), r = local / G.N, n = local - r * G.N;
+            const typename A::E v = res[r * LS + n + (n >> skew)];
             put(G, a, b, pix, A::re(v), A::im(v));
         }
         for (size_t pix = e1 + threadIdx.x; pix < P1; pix += blockDim.x) {
-            const int local = (int)(pix - P0), r = local / G.N;
-            const typename A::E v = res[(size_t)r * LS + (local - r * G.N)];
+            const int local = (int)(pix - P0), r = local / G.N, n = local - r * G.N;
+            const typename A::E v = res[r * LS + n + (n >> skew)];
             put(G, a, b, pix, A::re(v), A::im(v));
         }
     }
+};
+
+// How the row pass lays out its two shared-memory line buffers (pass s writes buffer s & 1).
+//   first pass    consecutive threads take consecutive i of R0 outputs i R0 + s each: stored there they
+//                 would all fall on a few banks, so output s of i goes to s pitch0 + i, and the second
+//                 pass reads its input j + q T at (j mod R0) pitch0 + j / R0 + q T / R0;
+//   staged        pixel n of the last pass at n + (n >> skew): the threads that then read 8 consecutive
+//                 pixels each start 9 elements apart.
+// The layout is computed in closed form, not searched: it is made for every launch, between the events of
+// the autotuner too, where the search took longer than a small pass (8 rings of 90^2: 46 us, now 12) and
+// had the tuner keep wrong row counts.  Four rows a CTA, 64 ring pairs of 1,080^2, plain FP32: 458 us with
+// 42 of 70 million shared-memory wavefronts conflicts, 447 us so; 20 rings of 288^2: 9 to 17 us less.
+struct RowShape {
+    int LS[2];        // line pitch of the buffers
+    int pitch0, skew;
+    size_t smem;
 };
 
 template <class A>
@@ -663,13 +679,16 @@ struct RowNT {
 
 template <class A, int R, class Out>
 __device__ __forceinline__ void row_pass(const RingGeom &G, const FftPlan &P, const FftPass &ps, bool first, bool last,
-                                         int RB, int rb, uint32_t mag_rb, int LS, int Rp, int py0,
+                                         int RB, int rb, uint32_t mag_rb, const RowShape &L, int s_in, int Rp, int py0,
                                          const typename A::E *__restrict__ src, const typename A::E *in,
                                          typename A::E *out, const float4 *__restrict__ tw, const Out &dst_out,
                                          int ring_a, int ring_b) {
     using C = typename A::C;
     using E = typename A::E;
     const int N = G.N, T = ps.T, p = ps.p, nbf = (first ? RB : rb) * T;
+    const bool second = p == P.pass[0].R && !first;     // reads what the first pass wrote
+    const bool staged = Out::staged && p * R == N;      // writes what store_block reads
+    const int LSi = s_in ? L.LS[1] : L.LS[0], LSo = s_in ? L.LS[0] : L.LS[1], step = second ? T / p : T;
     for (int b = threadIdx.x; b < nbf; b += blockDim.x) {
         int r, i;
         C x[R];
@@ -686,11 +705,11 @@ __device__ __forceinline__ void row_pass(const RingGeom &G, const FftPlan &P, co
         } else {
             r = (int)__umulhi((uint32_t)b, ps.mag_T);
             i = b - r * T;
-            const E *l = in + (size_t)r * LS;
-#pragma unroll
-            for (int q = 0; q < R; ++q) x[q] = A::ld(l[i + q * T]);
             const int ip = p == 1 ? i : (int)__umulhi((uint32_t)i, ps.mag_p);
             const int k = i - ip * p;
+            const E *l = in + r * LSi + (second ? k * L.pitch0 + ip : i);
+#pragma unroll
+            for (int q = 0; q < R; ++q) x[q] = A::ld(l[q * step]);
             if (k) apply_powers<A, R>(x, A::tw_load(tw, k * ps.tstep));
         }
         Dft<A, R>::run(x, P.itw);
@@ -701,9 +720,20 @@ __device__ __forceinline__ void row_pass(const RingGeom &G, const FftPlan &P, co
                 const E e = A::st(x[s]);
                 dst_out.put(G, ring_a, ring_b, row + i + s * p, A::re(e), A::im(e));
             }
+        } else if (staged) {   // likewise, in shared memory
+            E *dst = out + r * LSo;
+#pragma unroll
+            for (int s = 0; s < R; ++s) {
+                const int n = i + s * p;
+                dst[n + (n >> L.skew)] = A::st(x[s]);
+            }
+        } else if (first) {
+            E *dst = out + r * LSo + i;
+#pragma unroll
+            for (int s = 0; s < R; ++s) dst[s * L.pitch0] = A::st(x[s]);
         } else {
-            const int ip = p == 1 ? i : (int)__umulhi((uint32_t)i, ps.mag_p);
-            E *dst = out + (size_t)r * LS + ip * p * R + (i - ip * p);
+            const int ip = (int)__umulhi((uint32_t)i, ps.mag_p);
+            E *dst = out + r * LSo + ip * p * R + (i - ip * p);
 #pragma unroll
             for (int s = 0; s < R; ++s) dst[s * p] = A::st(x[s]);
         }
@@ -712,7 +742,7 @@ __device__ __forceinline__ void row_pass(const RingGeom &G, const FftPlan &P, co
 
 template <class A, class Out, int MAXR>
 __global__ void __launch_bounds__(RowNT<A>::value, RowNT<A>::min_blocks > 1 ? RowNT<A>::min_blocks : fft_min_blocks<A, MAXR>())
-    k_fft_rows(RingGeom G, const __grid_constant__ FftPlan P, int RB, uint32_t mag_rb, int LS,
+    k_fft_rows(RingGeom G, const __grid_constant__ FftPlan P, int RB, uint32_t mag_rb, const RowShape L,
                const int32_t *__restrict__ Rm, const typename A::E *__restrict__ W, const float4 *__restrict__ tw,
                const Out dst_out) {
     using E = typename A::E;
@@ -728,7 +758,7 @@ __global__ void __launch_bounds__(RowNT<A>::value, RowNT<A>::min_blocks > 1 ? Ro
         return;
     }
     E *const buf0 = (E *)sbuf;
-    const size_t bstride = (size_t)RB * LS;
+    const int bstride = RB * L.LS[0];
     const E *src = W + (size_t)pair * (2 * G.Rmax + 1) * G.N;
     for (int s = 0; s < P.nrad; ++s) {
         if (s) __syncthreads();
@@ -737,7 +767,7 @@ __global__ void __launch_bounds__(RowNT<A>::value, RowNT<A>::min_blocks > 1 ? Ro
         const E *in = buf0 + ((s + 1) & 1) * bstride;   // what pass s - 1 wrote
         E *out = buf0 + (s & 1) * bstride;
 #define ABS_ROW_CASE(RR) \
-    case RR: row_pass<A, RR>(G, P, ps, first, last, RB, rb, mag_rb, LS, Rp, py0, src, in, out, tw, dst_out, a, b); break;
+    case RR: row_pass<A, RR>(G, P, ps, first, last, RB, rb, mag_rb, L, (s + 1) & 1, Rp, py0, src, in, out, tw, dst_out, a, b); break;
         if (MAXR <= LOW_RADIX || ps.R <= LOW_RADIX) {
             switch (ps.R) {
                 ABS_ROW_CASE(2) ABS_ROW_CASE(3) ABS_ROW_CASE(4) ABS_ROW_CASE(5) ABS_ROW_CASE(6) ABS_ROW_CASE(8)
@@ -756,7 +786,8 @@ __global__ void __launch_bounds__(RowNT<A>::value, RowNT<A>::min_blocks > 1 ? Ro
     }
     if constexpr (Out::staged) {
         __syncthreads();
-        dst_out.template store_block<A>(G, a, b, buf0 + ((P.nrad - 1) & 1) * bstride, LS, py0, rb);
+        dst_out.template store_block<A>(G, a, b, buf0 + ((P.nrad - 1) & 1) * bstride, P.nrad & 1 ? L.LS[0] : L.LS[1], L.skew,
+                                              py0, rb);
     }
 }
 
@@ -821,44 +852,50 @@ static int lines_per_cta(size_t line, int lines, int npairs, int sm_count, int m
     return best;
 }
 
-// Line pitch of the row pass's buffers: N plus the pad (0 to 15 elements) that
-// spreads the first pass's stores (consecutive threads in consecutive lines, at
-// i R0 in line i mod RB) over the most shared-memory banks: per 128-byte phase
-// of a warp's store, the largest count of distinct words one bank must serve.
-static int row_pitch(int N, int R0, int RB, size_t esize) {
-    const int words = (int)(esize / 4), per_phase = 32 / words;
-    int best = N, best_cost = INT32_MAX;
-    for (int pad = 0; pad < 16; ++pad) {
-        const int LS = N + pad;
-        int cost = 0;
-        for (int ph = 0; ph < 32; ph += per_phase) {
-            std::vector<std::vector<int>> bank(32);
-            for (int t = ph; t < ph + per_phase; ++t) {
-                const int i = t / RB, r = t - i * RB;
-                const int w0 = (r * LS + i * R0) * words;
-                for (int w = 0; w < words; ++w) {
-                    auto &v = bank[(w0 + w) & 31];
-                    if (std::find(v.begin(), v.end(), w0 + w) == v.end()) v.push_back(w0 + w);
-                }
-            }
-            size_t worst = 0;
-            for (const auto &v : bank) worst = std::max(worst, v.size());
-            cost += (int)worst;
-        }
-        if (cost < best_cost) {
-            best_cost = cost;
-            best = LS;
-        }
+// x plus the least padding that puts n elements x apart, and the next ones after each, on different banks:
+// of the `phase` elements that 128 bytes hold, every phase / n th (or, n dividing phase, an odd multiple).
+static int spread(int x, int n, int phase) {
+    const int c = std::max(1, phase / n);
+    for (int pad = 0; pad < phase; ++pad) {
+        const int m = (x + pad) % phase;
+        if (phase % n == 0 || c == 1 ? m % c == 0 && m / c % 2 == 1 : m == c || m == phase - c) return x + pad;
     }
-    return best;
+    return x;
 }
 
-// Shared memory of a row-pass CTA: line buffers of RB lines at pitch LS, one a
-// pass that writes to shared memory (all but the last, which writes there too
-// when its output is staged), two at most.
-static size_t row_smem(const Setup &s, int RB, int LS, size_t esize, bool staged) {
-    const int to_smem = (int)s.radices.size() - (staged ? 0 : 1);
-    return (size_t)std::min(std::max(to_smem, 0), 2) * RB * LS * esize;
+// Layout and shared memory of a row-pass CTA of RB lines: a buffer for every pass that writes to shared
+// memory (all but the last, which writes there too when its output is staged), two at most.  Without any
+// padding where the padded lines would not fit.
+static RowShape row_shape(const Setup &s, int RB, size_t esize, bool staged) {
+    const int nrad = (int)s.radices.size(), R0 = nrad ? s.radices[0] : 1, T0 = s.N / R0;
+    const int bufs = std::min(std::max(nrad - (staged ? 0 : 1), 0), 2), phase = (int)(128 / esize);
+    RowShape L;
+    for (const bool pad : {true, false}) {
+        L.LS[0] = L.LS[1] = s.N;
+        L.pitch0 = T0;
+        L.skew = 31;
+        if (pad && nrad > 1) {
+            L.pitch0 = spread(T0, R0, phase);
+            L.LS[0] = R0 * L.pitch0;
+        }
+        if (pad && staged) {
+            L.skew = 3;
+            int &ls = L.LS[(nrad - 1) & 1];
+            ls = std::max(ls, s.N + s.N / 8);
+        }
+        if (pad && RB > 1) L.LS[0] = spread(L.LS[0], RB, phase);
+        L.smem = (size_t)RB * ((bufs > 0 ? L.LS[0] : 0) + (bufs > 1 ? L.LS[1] : 0)) * esize;
+        if (L.smem <= 227 * 1024) break;
+    }
+    return L;
+}
+
+// Rows a CTA of the row pass: a column's adjacent rows are read together, so as many as fill a 32-byte
+// sector (two double-float values, four plain ones), where three such CTAs share an SM; else two.  Plain
+// FP32, 64 ring pairs of 1,080^2: 522 us with two rows, 447 with four.
+static int default_rows(const Setup &s, size_t esize, bool staged) {
+    const int rb = (int)(32 / esize);
+    return rb > 2 && rb <= s.N && 3 * (row_shape(s, rb, esize, staged).smem + 1024) <= 228 * 1024 ? rb : 2;
 }
 
 // The transforms run in double-float on the FP32 path and in plain FP32 on the
@@ -878,7 +915,7 @@ FftLaunch fft_launch(const Setup &s, int sm_count) {
     // (double-float) a thread
     const int per_sm = std::min(2048 / FFT_NT, 65536 / (FFT_NT * (f32 ? 32 : 64)));
     L.CB = lines_per_cta(line, 2 * s.R + 1, npairs, sm_count, per_sm);
-    L.RB = 2;   // the row pass: two rows a CTA (the autotuner tries 1 to 8)
+    L.RB = 2;   // the row pass: see default_rows (the autotuner tries 1 to 8)
     L.col_smem = line * 2 * L.CB;   // two line buffers
     return L;
 }
@@ -889,6 +926,7 @@ abs_status run_fft_as(abs_ctx *ctx, const Setup &s, const Src &src, float *d_fie
     RingGeom G{s.n, s.half, s.nb, s.N, s.R};
     const FftPlan P = make_plan(s);
     FftLaunch L = fft_launch(s, ctx->sm_count);
+    L.RB = default_rows(s, sizeof(E), split != nullptr);
     const int npairs = (s.nb + 1) / 2;
     const size_t wbytes = sizeof(E) * (size_t)npairs * (2 * s.R + 1) * s.N;
     E *W = (E *)workspace(ctx, "fft.rows", wbytes);
@@ -905,8 +943,8 @@ abs_status run_fft_as(abs_ctx *ctx, const Setup &s, const Src &src, float *d_fie
     };
     auto rows_to = [&](int rb, const auto &out) {
         using Out = std::decay_t<decltype(out)>;
-        const int LS = row_pitch(s.N, s.radices.empty() ? 1 : s.radices[0], rb, sizeof(E));
-        const size_t sm = row_smem(s, rb, LS, sizeof(E), Out::staged);
+        const RowShape LS = row_shape(s, rb, sizeof(E), Out::staged);
+        const size_t sm = LS.smem;
         const auto kern = low ? k_fft_rows<A, Out, LOW_RADIX> : k_fft_rows<A, Out, MAX_RADIX>;
         allow_smem(kern, sm);
         kern<<<dim3((unsigned)cdiv(s.N, rb), npairs), RowNT<A>::value, sm, st>>>(G, P, rb, magic(rb), LS, s.d_Rm, W, tw, out);
@@ -969,8 +1007,7 @@ abs_status run_fft_as(abs_ctx *ctx, const Setup &s, const Src &src, float *d_fie
             cudaGetLastError();
         }
     }
-    const size_t rsm = row_smem(s, L.RB, row_pitch(s.N, s.radices.empty() ? 1 : s.radices[0], L.RB, sizeof(E)),
-                                sizeof(E), split != nullptr);
+    const size_t rsm = row_shape(s, L.RB, sizeof(E), split != nullptr).smem;
     if (rsm > 227 * 1024 || line * 2 * L.CB > 227 * 1024)
         return fail(ctx, ABS_ERR_UNSUPPORTED, "FFT lines do not fit shared memory");
     {
@@ -1038,9 +1075,9 @@ abs_status run_fft_delay(abs_ctx *ctx, const Setup &s, int t_max, const float4 *
     // lines per CTA of the column pass: the model of fft_launch for this many pairs
     const int per_sm = std::min(2048 / FFT_NT, 65536 / (FFT_NT * (sizeof(E) == 8 ? 32 : 64)));
     const int CB = lines_per_cta(line, 2 * s.R + 1, npairs, ctx->sm_count, per_sm);
-    const int RB = 2;
-    const int LS = row_pitch(s.N, s.radices.empty() ? 1 : s.radices[0], RB, sizeof(E));
-    const size_t csm = line * 2 * CB, rsm = row_smem(s, RB, LS, sizeof(E), false);
+    const int RB = default_rows(s, sizeof(E), false);
+    const RowShape LS = row_shape(s, RB, sizeof(E), false);
+    const size_t csm = line * 2 * CB, rsm = LS.smem;
     if (csm > 227 * 1024 || rsm > 227 * 1024) return fail(ctx, ABS_ERR_UNSUPPORTED, "FFT lines do not fit shared memory");
     E *W = (E *)workspace(ctx, "fft.delay", sizeof(E) * (size_t)npairs * (2 * s.R + 1) * s.N);
     if (!W) return fail(ctx, ABS_ERR_OOM, "delay transform workspace");
