@@ -8,7 +8,7 @@
 // Plan (per baseline set): key every visibility by its 16x16-cell uv tile and
 // its cell in the tile and stable-sort positions and original indices by that
 // key (LSD radix, two passes up to about 500^2 cells, three beyond); the
-// sorted order is cut into work units of UMAX records.
+// sorted order is cut into work units of UMAX records (fewer for small sets, see grid_unit).
 //
 // Accumulation (per realisation): one CTA per unit stages the unit in shared
 // memory, forms the 1-D Gaussian weights and cuts it into runs of
@@ -379,7 +379,7 @@ ScatterFn scatter_of(int dw, bool first, bool last) {
 }
 
 // ------------------------------------------------------------------ accumulation
-// One CTA per work unit: UMAX consecutive visibilities of the sorted order,
+// One CTA per work unit: um consecutive visibilities (at most UMAX) of the sorted order,
 // so a unit's visibilities come grouped by cell (any number of cells and
 // tiles).  Each visibility's 2 (2r+1) one-dimensional weights are formed
 // once and staged in shared memory, and the unit is cut into tasks: runs of
@@ -447,24 +447,24 @@ __device__ __forceinline__ void grid_acc(const float *lw, const float *lwy, cons
     if (WM == GW_SUM_SQ) ws2 = __ffma2_rn(w, w, ws2);
 }
 
-// Inputs of one unit as thread (warp, lane) sees them: items t = 64 warp +
-// 32 h + lane, h = 0, 1, in sorted order.
+// Inputs of one unit as thread (warp, lane) sees them: items t = ipw warp +
+// 32 h + lane, h = 0, 1 (h = 0 only when ipw is 32), in sorted order.
 struct UnitIn {
     int cnt;
     float2 p[2];
     uint32_t idx[2];
 };
 
-__device__ __forceinline__ void load_unit(UnitIn &in, int64_t u, int64_t nu, int64_t n_vis,
+__device__ __forceinline__ void load_unit(UnitIn &in, int64_t u, int64_t nu, int64_t n_vis, int um, int ipw,
                                           const float2 *__restrict__ s_uv, const uint32_t *__restrict__ s_idx,
                                           int warp, int lane) {
     if (u >= nu) return;
-    const int64_t b = u * UMAX;
-    in.cnt = n_vis - b < UMAX ? (int)(n_vis - b) : UMAX;
+    const int64_t b = u * um;
+    in.cnt = n_vis - b < um ? (int)(n_vis - b) : um;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const int t = warp * 64 + h * 32 + lane;
-        if (t < in.cnt) {
+        const int t = warp * ipw + h * 32 + lane;
+        if (h * 32 < ipw && t < in.cnt) {
             in.p[h] = s_uv[b + t];
             in.idx[h] = s_idx[b + t];
         }
@@ -491,7 +491,7 @@ __device__ __forceinline__ void grid_add(double *__restrict__ re, double *__rest
 }
 
 template <int WM>
-__global__ void __launch_bounds__(GT, 3) k_grid(GridGeom G, int64_t n_vis, uint32_t key_none,
+__global__ void __launch_bounds__(GT, 3) k_grid(GridGeom G, int64_t n_vis, int um, uint32_t key_none,
                                              const float2 *__restrict__ s_uv,
                                              const uint32_t *__restrict__ s_idx,
                                              const float2 *__restrict__ vis,
@@ -511,27 +511,28 @@ __global__ void __launch_bounds__(GT, 3) k_grid(GridGeom G, int64_t n_vis, uint3
     // this lane's footprint cells: (qx, dy) and (qx + 4, dy)
     const int dy = lane >> 2, qx = lane & 3;
     const bool on_a = dy < fw && qx < fw, on_b = on_a && qx + 4 < fw;
-    const int64_t nu = cdiv(n_vis, UMAX);
+    const int ipw = um > GT ? 64 : 32;   // items a warp
+    const int64_t nu = cdiv(n_vis, um);
     UnitIn nxt;
-    load_unit(nxt, blockIdx.x, nu, n_vis, s_uv, s_idx, warp, lane);
+    load_unit(nxt, blockIdx.x, nu, n_vis, um, ipw, s_uv, s_idx, warp, lane);
     float2 vn[2];   // the next unit's visibilities, gathered one unit ahead
 #pragma unroll
     for (int h = 0; h < 2; ++h)
-        if (blockIdx.x < nu && warp * 64 + h * 32 + lane < nxt.cnt) vn[h] = vis[nxt.idx[h]];
+        if (blockIdx.x < nu && h * 32 < ipw && warp * ipw + h * 32 + lane < nxt.cnt) vn[h] = vis[nxt.idx[h]];
     for (int64_t u = blockIdx.x; u < nu; u += gridDim.x) {
         const UnitIn cur = nxt;
         const int total = cur.cnt;
         const float2 v[2] = {vn[0], vn[1]};   // this unit's visibilities
-        load_unit(nxt, u + gridDim.x, nu, n_vis, s_uv, s_idx, warp, lane);   // in flight during this unit
+        load_unit(nxt, u + gridDim.x, nu, n_vis, um, ipw, s_uv, s_idx, warp, lane);   // in flight during this unit
         __syncthreads();   // previous unit done with the staging buffers
         // keys (the plan's, recomputed from the same positions); invalid items sort last
         float2 q[2];   // u/dU, v/dU of this thread's items
         bool valid[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int t = warp * 64 + h * 32 + lane;
+            const int t = warp * ipw + h * 32 + lane;
             valid[h] = false;
-            if (t < total) {
+            if (h * 32 < ipw && t < total) {
                 q[h] = quotients(G, cur.p[h]);
                 const uint32_t key = key_from_q(G, q[h], key_none);
                 skey[t] = key;
@@ -543,7 +544,7 @@ __global__ void __launch_bounds__(GT, 3) k_grid(GridGeom G, int64_t n_vis, uint3
         bool ts[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int t = warp * 64 + h * 32 + lane;
+            const int t = warp * ipw + h * 32 + lane;
             ts[h] = valid[h] && (t % CHUNK == 0 || skey[t] != skey[t - 1]);
         }
         const unsigned b0 = __ballot_sync(FULL, ts[0]), b1 = __ballot_sync(FULL, ts[1]);
@@ -561,8 +562,8 @@ __global__ void __launch_bounds__(GT, 3) k_grid(GridGeom G, int64_t n_vis, uint3
             nvalid += wvalid_s[w];
         }
         const unsigned lt = (1u << lane) - 1u;
-        if (ts[0]) tstart[wbase + __popc(b0 & lt)] = (uint16_t)(warp * 64 + lane);
-        if (ts[1]) tstart[wbase + __popc(b0) + __popc(b1 & lt)] = (uint16_t)(warp * 64 + 32 + lane);
+        if (ts[0]) tstart[wbase + __popc(b0 & lt)] = (uint16_t)(warp * ipw + lane);
+        if (ts[1]) tstart[wbase + __popc(b0) + __popc(b1 & lt)] = (uint16_t)(warp * ipw + 32 + lane);
         if (threadIdx.x == 0) {
             tstart[ntask] = (uint16_t)nvalid;
             next_s = GT / 32;   // the warps' first tasks are their own numbers
@@ -570,7 +571,7 @@ __global__ void __launch_bounds__(GT, 3) k_grid(GridGeom G, int64_t n_vis, uint3
         // staging: weights and visibility of every valid item, in place
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int t = warp * 64 + h * 32 + lane;
+            const int t = warp * ipw + h * 32 + lane;
             if (valid[h]) {
                 const float2 p = cur.p[h], qq = q[h];
                 const float cxf = floorf(__fadd_rn(qq.x, 0.5f)), cyf = floorf(__fadd_rn(qq.y, 0.5f));
@@ -599,7 +600,7 @@ __global__ void __launch_bounds__(GT, 3) k_grid(GridGeom G, int64_t n_vis, uint3
         // the next unit's visibilities: its indices have arrived by now
 #pragma unroll
         for (int h = 0; h < 2; ++h)
-            if (u + gridDim.x < nu && warp * 64 + h * 32 + lane < nxt.cnt) vn[h] = vis[nxt.idx[h]];
+            if (u + gridDim.x < nu && h * 32 < ipw && warp * ipw + h * 32 + lane < nxt.cnt) vn[h] = vis[nxt.idx[h]];
         __syncthreads();
         for (int tk = warp, nx = 0; tk < (int)ntask; tk = nx) {
             if (lane == 0) nx = atomicAdd(&next_s, 1);   // tasks differ in length: the next free one
@@ -758,6 +759,17 @@ void grid_acc_buffers(abs_ctx *ctx, const Setup &s, double **acc) {
     *acc = (double *)workspace(ctx, "grid.acc", sizeof(double) * grid_acc_planes(s) * cells);
 }
 
+// Visibilities of a gridding unit: UMAX where that gives every resident CTA a unit, else half or a quarter
+// of it (a unit is a chain of staging and sums, and on a small set the longest one is the kernel).  All are
+// multiples of CHUNK, so the runs, and with them the results, are the same.
+// 5,000 visibilities on 64^2: 27 us with 512 a unit, 12 with 128; 50,000 on 256^2: 35 / 20; 80,000 on 512^2:
+// 55 / 36; 160,000 (256 a unit): 59 / 52; equal from 230,000 on.
+static int grid_unit(int64_t n_vis, int ctas) {
+    int um = UMAX;
+    while (um > CHUNK && cdiv(n_vis, um) < ctas) um /= 2;
+    return um;
+}
+
 abs_status launch_grid_accumulate(abs_ctx *ctx, const Setup &s, int64_t n_vis, const float *d_vis,
                                   float *d_grid, float *d_wsum, uint8_t *d_mask, bool acc_zeroed, abs_ctx *plan) {
     // the estimate path (no FP32 outputs; its plan was made with rings_only) accumulates what
@@ -780,10 +792,11 @@ abs_status launch_grid_accumulate(abs_ctx *ctx, const Setup &s, int64_t n_vis, c
     }
     if (n_vis > 0) {
         StageTimer timer(ctx, "grid");
-        const int blocks = (int)std::min<int64_t>(cdiv(n_vis, UMAX), ctx->sm_count * 3);
+        const int um = grid_unit(n_vis, ctx->sm_count * 3);
+        const int blocks = (int)std::min<int64_t>(cdiv(n_vis, um), ctx->sm_count * 3);
         auto run = [&](auto kern) {
             allow_smem(kern, GRID_SMEM);
-            kern<<<blocks, GT, GRID_SMEM, st>>>(G, n_vis, plan_key_none(b), b.s_uv, b.s_idx, (const float2 *)d_vis,
+            kern<<<blocks, GT, GRID_SMEM, st>>>(G, n_vis, um, plan_key_none(b), b.s_uv, b.s_idx, (const float2 *)d_vis,
                                                 acc, acc + cells, acc + 2 * cells, acc + 3 * cells);
         };
         if (wm == GW_COUNT)

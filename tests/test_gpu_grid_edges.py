@@ -74,3 +74,10 @@ def test_runs_of_one_cell(kernel, sigma, radius):
         c = c[rng.permutation(len(c))]
     uv = ((c + rng.uniform(-0.5, 0.5, c.shape)) * 2.0).astype(np.float32)
     _check(n, 2.0, uv, _vis(rng, len(uv)), kernel, sigma, radius)
+
+
+@pytest.mark.parametrize("n_vis", [60_000, 120_001, 240_003])   # units of 128, 256 and 512 visibilities
+def test_units(n_vis):
+    rng = np.random.default_rng(n_vis)
+    uv = (rng.uniform(-0.5, 0.5, (n_vis, 2)) * 90).astype(np.float32)
+    _check(90, 1.0, uv, _vis(rng, n_vis))
