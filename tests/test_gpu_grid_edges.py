@@ -81,3 +81,12 @@ def test_units(n_vis):
     rng = np.random.default_rng(n_vis)
     uv = (rng.uniform(-0.5, 0.5, (n_vis, 2)) * 90).astype(np.float32)
     _check(90, 1.0, uv, _vis(rng, n_vis))
+
+
+@pytest.mark.parametrize("n_grid", [16, 66, 600])   # keys of two and of three passes
+@pytest.mark.parametrize("n_vis", [1023, 1025, 5119, 5120, 5121])   # rows and the largest set of the one-CTA plan
+def test_one_cta_plan(n_grid, n_vis):
+    rng = np.random.default_rng(n_vis + n_grid)
+    uv = (rng.uniform(-0.52, 0.52, (n_vis, 2)) * n_grid * 0.9).astype(np.float32)
+    uv[::97] = np.inf
+    _check(n_grid, 0.9, uv, _vis(rng, n_vis))
