@@ -318,7 +318,9 @@ def count_route_visits(A, F):
     """Pair visits of the exact count kernel, which takes the cheaper of its two routes: the
     direct enumeration of the filled cells, sum over a <= b of floor(F_a / 2) F_b, or the
     holes route (H = A - F), sum over a <= b of floor(H_a / 2) A_b + 2 floor(F_a / 2) H_b
-    (the full-annulus table it subtracts from is computed once per configuration)."""
+    (the full-annulus table it subtracts from is computed once per configuration).  The unit is
+    the plain enumeration: the kernel's holes route halves the one-hole terms and takes the
+    annulus by its symmetric orbits, so a rate in this unit is above its executed one."""
     H = A - F
     tail = lambda v: np.cumsum(v[::-1])[::-1]          # sum over b >= a
     direct = int(np.sum((F // 2) * tail(F)))

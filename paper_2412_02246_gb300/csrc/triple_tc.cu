@@ -28,35 +28,42 @@
 // takes items from a queue (one atomic counter), ranges outermost, so that the
 // sets that read the same pixels run at about the same time and share them in L2.
 //
-// Per 64-pixel chunk c of an item, three roles and their mbarriers:
+// Per 64-pixel chunk c of an item, four roles and their mbarriers:
 //   loader (warp 0)    bulk copies of chunk c into stage s = c mod n_stages:
 //                      the set's window of rings of the hi and lo planes (the
 //                      MMA operand B, K-major, 128-byte swizzle) and the window
 //                      of rings its rows form A from (FP32), counted on full[s];
 //                      it reuses stage s once done[s] says chunk c - n_stages has
 //                      finished with it;
-//   formers (warps 2..) thread = one row (its tensor-memory lane) and 64 / FQ
+//   formers (FW0 ..)   thread = one row (its tensor-memory lane) and 64 / FQ
 //                      of the 64 pixels (32 with eight forming warps), for every tile
 //                      of the set: A = D_j D_k in FP32, split, packed in BF16
 //                      pairs and stored to A buffer (c & 1) of the tile in
 //                      tensor memory (tcgen05.st); one arrival on a_full[c & 1]
 //                      a warp per chunk.  Buffer (c & 1) is free again once
 //                      done[] of chunk c - 2 has completed;
-//   MMA issuer (warp 1) per tile, 4 K-steps x 3 MMAs (A from tensor memory, B
+//   MMA issuers (1 ..) per tile, 4 K-steps x 3 MMAs (A from tensor memory, B
 //                      from the stage), M = 128, N = the tile's ring columns,
 //                      into accumulation region (g & 1) of group g = c / DRAIN;
 //                      one tcgen05.commit per chunk to done[s] (the stage and
 //                      the A buffers of chunk c are free), and at the end of
-//                      a group one to d_full[g & 1].
+//                      a group one to d_full[g & 1];
+//   drainers (DW0 ..)  add a complete group's region to long accumulators.
 // Tensor-core accumulation in FP32 over long pixel ranges loses accuracy (the
 // error grows with the number of chunks summed into one accumulator), so every
-// DRAIN chunks the formers read the group's region back (tcgen05.ld) into FP32
+// DRAIN chunks the drainers read the group's region back (tcgen05.ld) into FP32
 // registers, one long accumulator per (row, column) a thread owns, and release
 // it (d_empty); the issuer meanwhile fills the other region.  After the item's
-// last chunk the formers write the long accumulators, column-major by tile
+// last chunk the drainers write the long accumulators, column-major by tile
 // (lanes contiguous), to the item's pixel range of the partial-sum array.  A
 // second kernel adds the pixel ranges in double-float in a fixed order and gathers each
 // triplet's entry.
+//
+// What bounds it: the formers, eight warps each with a serial chain of loads, products,
+// splits and stores a tile (1.80 ms on 128 rings of 1,080^2, of which the MMAs alone take
+// 0.9; issue 49 %, ALU 43 %, the shared-memory data path 68 %).  Draining in warps of
+// their own took 0.1 ms off: the long accumulators, 64 registers a thread, had left the
+// formers spilling.
 //
 // Rates that shaped this design, measured on GB300 with microbenchmarks: an MMA
 // of M = 128, K = 16 costs max(45.5, N / 2) cycles of the tensor pipe, with A in
@@ -85,7 +92,7 @@ constexpr int KC = 64;               // pixels per chunk (4 MMA K-steps of 16)
 #ifndef ABS_TC_FORMERS
 #define ABS_TC_FORMERS 8
 #endif
-constexpr int NFORM = ABS_TC_FORMERS;   // forming / epilogue warps (8 or 16)
+constexpr int NFORM = ABS_TC_FORMERS;   // forming warps
 constexpr int FQ = NFORM / 4;           // forming warps per tensor-memory lane quadrant
 constexpr int FPX = KC / FQ;            // pixels of a chunk per forming thread
 #ifndef ABS_TC_MAX_TILES
@@ -124,7 +131,7 @@ constexpr int DRAIN = ABS_TC_DRAIN;  // chunks accumulated in tensor memory befo
 #define ABS_TC_SET_COLS 128
 #endif
 // accumulator columns of a set: two accumulation regions beside the A buffers fit tensor
-// memory up to 192; the forming threads' long accumulators (set columns / (4 FQ) each)
+// memory up to 192; the draining threads' long accumulators (set columns / DQ each)
 // bound it by registers
 constexpr int MAX_SET_COLS = ABS_TC_SET_COLS;
 static_assert(NABUF * A_COLS + 2 * MAX_SET_COLS <= TMEM_COLS, "A buffers and two regions fit tensor memory");
