@@ -211,15 +211,33 @@ abs_status launch_simulate_vis(abs_ctx *ctx, int32_t m, double dtheta, const flo
                                double beam_param, int64_t n_vis, const float *d_uv, float *d_vis) {
     const int64_t npix = (int64_t)m * m;
     float *W = (float *)workspace(ctx, "sim.weights", sizeof(float) * (size_t)npix);
+    if (!W) return fail(ctx, ABS_ERR_OOM, "simulator workspace");
     // column blocks and row ranges (whole staged passes) so that the launch holds about eight waves
-    // of CTAs, two to an SM by their registers; the visibilities in slabs whose parts take 256 MB at most
+    // of CTAs, two to an SM by their registers; the visibilities in slabs whose parts take `room` bytes at most
     const int ny = (int)cdiv(m, SIM_A);
-    const int64_t slab = std::min<int64_t>(n_vis, std::max<int64_t>(SIM_T * SIM_V, (((int64_t)256 << 20) / 16 / ny) / (SIM_T * SIM_V) * (SIM_T * SIM_V)));
-    const int64_t ctas = std::max<int64_t>(cdiv(slab, SIM_T * SIM_V) * ny, 1);
-    const int want = (int)std::min<int64_t>(cdiv(m, SIM_ROWS), cdiv((int64_t)16 * ctx->sm_count, ctas));
-    const int rows_per = (int)cdiv(cdiv(m, want), SIM_ROWS) * SIM_ROWS, nz = (int)cdiv(m, rows_per);
-    float4 *part = (float4 *)workspace(ctx, "sim.parts", sizeof(float4) * (size_t)(ny * nz) * slab);
-    if (!W || !part) return fail(ctx, ABS_ERR_OOM, "simulator workspace");
+    int64_t slab = 0;
+    int rows_per = 0, nz = 0;
+    auto shape = [&](int64_t room) {
+        const int64_t fit = room / (int64_t)sizeof(float4) / ny, unit = SIM_T * SIM_V;
+        slab = std::min<int64_t>(n_vis, std::max<int64_t>(fit < unit ? fit : fit / unit * unit, 1));
+        const int64_t ctas = std::max<int64_t>(cdiv(slab, unit) * ny, 1), most = slab > 0 ? std::max<int64_t>(fit / slab, 1) : 1;
+        const int want = (int)std::min(std::min<int64_t>(cdiv(m, SIM_ROWS), cdiv((int64_t)16 * ctx->sm_count, ctas)), most);
+        rows_per = (int)cdiv(cdiv(m, want), SIM_ROWS) * SIM_ROWS;
+        nz = (int)cdiv(m, rows_per);
+        return sizeof(float4) * (size_t)(ny * nz) * (size_t)slab;
+    };
+    // 256 MB, or as much as there is: less if the device has not the room, and what an earlier call left in a
+    // stream that is being captured, where nothing can be allocated
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &capturing) != cudaSuccess) cudaGetLastError();
+    const bool fixed = capturing != cudaStreamCaptureStatusNone;
+    const size_t have = ctx->ws["sim.parts"].bytes, least = sizeof(float4) * (size_t)ny;   // one visibility
+    size_t bytes = shape((int64_t)256 << 20);
+    if (fixed && bytes > have && have >= least) bytes = shape((int64_t)have);
+    float4 *part = (float4 *)workspace(ctx, "sim.parts", bytes);
+    for (size_t room = bytes / 2; !part && !fixed && room >= least; room /= 2)
+        part = (float4 *)workspace(ctx, "sim.parts", shape((int64_t)room));
+    if (!part) return fail(ctx, ABS_ERR_OOM, "simulator workspace");
     StageTimer timer(ctx, "simulate_vis");
     k_sky_weights<<<(unsigned)cdiv(npix, 256), 256, 0, ctx->stream>>>(m, dtheta, d_sky, beam, beam_param, W);
     for (int64_t v0 = 0; v0 < n_vis; v0 += slab) {
