@@ -439,6 +439,11 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
         const int f_bytes = S.f_n * 256;              // the F window (FP32 rows)
         const uint32_t tx_bytes = (uint32_t)(2 * b_bytes + f_bytes);
         const int region_cols = sum_n;
+        // a whole warp's wait: one answer for all its lanes, which stay together for the collective
+        // (.sync.aligned) instructions that follow
+        auto wait = [&](const uint64_t *bar, int parity) {
+            return __all_sync(FULL, mbar_wait(smem_u32(bar), (uint32_t)parity, &abort_s)) != 0;
+        };
 
         if (warp == 0) {
             // ---------------- loader
@@ -482,9 +487,6 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
             const uint64_t d_base = desc_sw128(uni(smem_u32(smem)));
             uint64_t d_cur = d_base + (uint64_t)st * d_stage;   // this chunk's stage, B hi plane
             int gc = 0;                                          // chunk in the group
-            auto wait = [&](const uint64_t *bar, int parity) {
-                return __all_sync(FULL, mbar_wait(smem_u32(bar), (uint32_t)parity, &abort_s)) != 0;
-            };
             for (int c = 0; c < nchunks; ++c) {
                 const uint32_t region = (uint32_t)(NABUF * A_COLS) + (grp & 1) * cols;
                 bool ok = true;
@@ -552,18 +554,18 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
             }
             bool fail_f = false;
             // a barrier test takes over 100 cycles to answer, so the next chunk's two are asked for before the
-            // end of this one: the copies have landed; the MMAs that read the next chunk's A slot are done
+            // end of this one: the copies have landed; the MMAs that read the next chunk's A slot are done.  A
+            // phase may complete between two lanes' tests: the warp goes on where all of them have seen it
             bool full_ok = false, done_ok = false;
             for (int c = 0; c < nchunks; ++c) {
-                if (!full_ok && !mbar_wait(smem_u32(&full[st]), (uint32_t)(su & 1), &abort_s)) {
+                if (!__all_sync(FULL, full_ok) && !wait(&full[st], su & 1)) {
                     fail_f = true;
                     break;
                 }
                 // the F window
                 const uint8_t *F = smem + (size_t)st * G.stage_bytes + 2 * b_bytes;
                 // the A buffers of this chunk's pair were read by the MMAs of chunk cg - 2
-                if (!done_ok && cg >= ASLOTS &&
-                    !mbar_wait(smem_u32(&done[hst[0]]), (uint32_t)(hsu[0] & 1), &abort_s)) {
+                if (!__all_sync(FULL, done_ok) && cg >= ASLOTS && !wait(&done[hst[0]], hsu[0] & 1)) {
                     fail_f = true;
                     break;
                 }
@@ -607,6 +609,7 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
                     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&a_full[(cg & (ASLOTS - 1)) * MAX_TILES + t]));
+                    __syncwarp();
                 }
                 // tiles the set does not have: their barriers keep step with the chunks
                 if (lane == 0)
@@ -629,7 +632,7 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
 #pragma unroll
             for (int x = 0; x < MAXSLOT; ++x) accl[x] = 0.f;
             for (int c = 0; c < nchunks; c += DRAIN) {
-                if (!mbar_wait(smem_u32(&d_full[grp & 1]), (uint32_t)((grp >> 1) & 1), &abort_s)) {
+                if (!wait(&d_full[grp & 1], (grp >> 1) & 1)) {
                     fail_f = true;
                     break;
                 }
