@@ -35,8 +35,10 @@
  * Ownership and execution: the caller allocates every d_* buffer on the
  * context's device and keeps it alive until the context's stream has
  * finished the call.  The context owns its workspaces, tables and caches and
- * frees them in abs_destroy.  All device work is enqueued asynchronously on
- * the context's stream.  A call returns ABS_OK once its work is enqueued, an
+ * frees them in abs_destroy.  A graph that the caller captures from a call
+ * holds the workspaces' addresses: it is valid until a later call on the
+ * context needs larger ones (or finds no room for them).  All device work is
+ * enqueued asynchronously on the context's stream.  A call returns ABS_OK once its work is enqueued, an
  * error code for bad arguments (nothing enqueued), or ABS_ERR_CUDA for a
  * launch failure.  Data-dependent device errors (for instance an unsorted
  * triplet list) are latched into the context and reported by abs_sync.
@@ -180,7 +182,13 @@ abs_status abs_estimate(abs_ctx *ctx, const abs_config *cfg, int64_t n_vis, cons
 /* abs_estimate on n_real realisations observed with the same baselines (the
  * ensemble of Sec. 3): d_vis [n_real][n_vis][2] float32, d_B [n_real][n_trip],
  * d_count [n_trip] (counts depend on the baselines only), d_ellbar [n_bins].
- * The baseline plan, the ring tables and the counts are built once. */
+ * The baseline plan, the ring tables and the counts are built once.  On a
+ * non-default stream the realisations run round-robin over the context's stream
+ * and its four lanes (see abs_estimate_batched) where one takes at most 512 MB
+ * of accumulators and fields (unweighted form; not for a caller's list in
+ * split-BF16).  The lanes keep their workspaces, up to 1.3 GB each at that
+ * size, for later calls; they are given back when a lane finds no room for a
+ * workspace (its realisations then run on the context's stream). */
 abs_status abs_estimate_many(abs_ctx *ctx, const abs_config *cfg, int64_t n_vis,
                              const float *d_uv, int32_t n_real, const float *d_vis,
                              int32_t n_trip, const int32_t *d_ijk, double *d_B,
@@ -369,9 +377,9 @@ abs_status abs_autotune(abs_ctx *ctx, int32_t enable);
 abs_status abs_probe_timeout(abs_ctx *ctx, int32_t max_polls);
 
 /* Failure injection on the host: the next `count` workspace allocations of the
- * context fail as if the device were out of memory (no device call is made
- * for them), so the calls that need them return ABS_ERR_OOM; later calls
- * allocate normally.  count >= 0 (0 turns it off). */
+ * context and its lanes fail as if the device were out of memory (no device
+ * call is made for them), so the calls that need them return ABS_ERR_OOM or do
+ * with less; later calls allocate normally.  count >= 0 (0 turns it off). */
 abs_status abs_inject_alloc_failures(abs_ctx *ctx, int32_t count);
 abs_status abs_tuned_shape(abs_ctx *ctx, const abs_config *cfg, int32_t *set_cols, int32_t *waves,
                            int32_t *measured);

@@ -56,6 +56,7 @@ struct Setup {
     // realisations of this configuration have been through lanes 0 .. lanes_ready - 1 (their workspaces
     // exist) with lists of lanes_trip triplets
     mutable int32_t lanes_ready = 0, lanes_trip = 0;
+    mutable bool lanes_refused = false;   // a lane found no room for its workspaces: not tried again
     // ordered closed-triangle counts of the full annuli [nb][nb][nb] (halved),
     // a property of the ring geometry, computed on first use
     unsigned long long *d_full_counts = nullptr;
@@ -134,7 +135,7 @@ struct abs_ctx {
     // autotuner: launch shapes of the split-BF16 kernel measured on a configuration's
     // first eager call, by configuration key; kept by the root context (lanes share it)
     bool autotune = true;
-    int32_t fail_allocs = 0;         // test hook: this many workspace allocations fail next
+    int32_t fail_allocs = 0;         // test hook: this many workspace allocations fail next (of the lanes too)
     // split-BF16 launch shape. budget: accumulator columns per set; waves: work items
     // per CTA (pixel ranges x sets / SMs)
     struct TcShape { bool measured = false; int budget = 0; int waves = 0; };
@@ -151,7 +152,8 @@ namespace absk {
 
 // Concurrent lanes of abs_estimate_batched (items round-robin over them).
 constexpr int ABS_BATCH_LANES = 4;
-// Largest realisation (accumulators and fields, bytes) that estimates of several run on lanes.
+// Largest realisation (accumulators and fields, bytes) that estimates of several run on lanes (a lane's
+// workspaces take up to 1.3 GB there).
 constexpr size_t LANE_REAL_BYTES = (size_t)512 << 20;
 // Creates lanes of ctx (child contexts with their own streams and workspaces, sharing its
 // device error word) until it has K.

@@ -239,6 +239,29 @@ void drop_graphs(abs_ctx *ctx) {
     if (ctx->parent) drop_graphs(ctx->parent);   // the parent's graphs hold this lane's buffers
 }
 
+// Gives the workspaces of ctx's lanes back to the device; false if they hold none, or while ctx's stream is
+// being captured.
+static bool release_lane_workspaces(abs_ctx *ctx) {
+    size_t held = 0;
+    for (abs_ctx *l : ctx->lanes)
+        for (auto &kv : l->ws) held += kv.second.bytes;
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &capturing) != cudaSuccess) cudaGetLastError();
+    if (!held || capturing != cudaStreamCaptureStatusNone) return false;
+    cudaStreamSynchronize(ctx->stream);
+    for (abs_ctx *l : ctx->lanes) {
+        cudaStreamSynchronize(l->stream);
+        cudaStreamSynchronize(l->side);
+    }
+    drop_graphs(ctx);
+    for (abs_ctx *l : ctx->lanes) {
+        for (auto &kv : l->ws) cudaFree(kv.second.p);
+        l->ws.clear();
+    }
+    for (auto &kv : ctx->setups) kv.second->lanes_ready = 0;
+    return true;
+}
+
 void *workspace(abs_ctx *ctx, const char *name, size_t bytes) {
     if (bytes == 0) bytes = 16;
     Workspace &w = ctx->ws[name];
@@ -251,15 +274,18 @@ void *workspace(abs_ctx *ctx, const char *name, size_t bytes) {
         w.bytes = 0;
     }
     const size_t want = bytes + bytes / 8;   // some headroom against regrowth
-    if (ctx->fail_allocs > 0) {              // injected failure (abs_inject_alloc_failures)
-        --ctx->fail_allocs;
-        return nullptr;
-    }
-    if (cudaMalloc(&w.p, want) != cudaSuccess) {
+    int32_t &failures = (ctx->parent ? ctx->parent : ctx)->fail_allocs;   // injected (abs_inject_alloc_failures)
+    auto allocate = [&] {
+        if (failures > 0) {
+            --failures;
+            return false;
+        }
+        if (cudaMalloc(&w.p, want) == cudaSuccess) return true;
         cudaGetLastError();
         w.p = nullptr;
-        return nullptr;
-    }
+        return false;
+    };
+    if (!allocate()) return nullptr;
     w.bytes = want;
     return w.p;
 }
@@ -814,10 +840,12 @@ static abs_status estimate_many(abs_ctx *ctx, const Setup &s, int64_t n_vis, con
     // workspaces of their own, forked from and joined back to it), the plan and the counts shared.  Eight
     // realisations on one stream / on five, FP32: 0.38 / 0.13 ms at 64^2 with 8 rings, 3.76 / 3.49 at 512^2
     // with 20, 55.4 / 48.8 at 1024^2 with 40 (360 MB each); split-BF16: 0.44 / 0.17, 2.41 / 2.11, 11.8 / 11.3.
-    // At 2048^2 with 20 rings (800 MB each) 107 / 106 ms no longer pay for five times the workspaces.  A
-    // caller's list in split-BF16 is planned on the host, one realisation after the other.
+    // At 2048^2 with 20 rings (800 MB each) 107 / 106 ms no longer pay for five times the workspaces.  The line
+    // counts accumulators and fields; a lane holds its transform rows (1.3 times the fields in double-float, a
+    // third of the planes in split-BF16) and up to some 0.1 GB of partial sums beside them.  A caller's list in
+    // split-BF16 is planned on the host, one realisation after the other.
     const size_t real_bytes = sizeof(double) * 3 * (size_t)cells + (size_t)s.nb * P * (to_planes ? 8 : 4);
-    int K = n_real > 1 && pre_zero && ctx->stream && !ctx->parent && !literal && real_bytes <= LANE_REAL_BYTES &&
+    int K = n_real > 1 && pre_zero && ctx->stream && !ctx->parent && !literal && !s.lanes_refused && real_bytes <= LANE_REAL_BYTES &&
                     (s.precision == ABS_FP32 || to_planes)
                 ? std::min<int>(ABS_BATCH_LANES, n_real - 1) : 0;
     // a stream that is being captured can make no lane and no workspace: lanes that an eager call with these
@@ -903,7 +931,11 @@ static abs_status estimate_many(abs_ctx *ctx, const Setup &s, int64_t n_vis, con
         if (l > 0 && lanes_on) {
             st = on_lane(r, ctx->lanes[l - 1]);
             if (st != ABS_OK && st != ABS_ERR_OOM) ctx->last_error = ctx->lanes[l - 1]->last_error;
-            lanes_on = st != ABS_ERR_OOM;   // no room for a lane's workspaces: the rest without lanes
+            if (st == ABS_ERR_OOM) {   // no room for a lane's workspaces: the rest, and later calls, without lanes
+                lanes_on = false;
+                s.lanes_refused = true;
+                release_lane_workspaces(ctx);   // the realisations queued on them end first
+            }
         }
         if (st == ABS_ERR_OOM) st = realisation(r);
         if (st != ABS_OK) return join_lanes(st);
