@@ -187,8 +187,9 @@ abs_status abs_estimate(abs_ctx *ctx, const abs_config *cfg, int64_t n_vis, cons
  * and its four lanes (see abs_estimate_batched) where one takes at most 512 MB
  * of accumulators and fields (unweighted form; not for a caller's list in
  * split-BF16).  The lanes keep their workspaces, up to 1.3 GB each at that
- * size, for later calls; they are given back when a lane finds no room for a
- * workspace (its realisations then run on the context's stream). */
+ * size, for later calls; they are given back when a lane or the context finds
+ * no room for a workspace (such a lane's realisations then run on the
+ * context's stream). */
 abs_status abs_estimate_many(abs_ctx *ctx, const abs_config *cfg, int64_t n_vis,
                              const float *d_uv, int32_t n_real, const float *d_vis,
                              int32_t n_trip, const int32_t *d_ijk, double *d_B,
@@ -220,8 +221,9 @@ typedef struct abs_item {
  * one CUDA graph on its second call with the same items (same
  * configurations and buffer addresses) and replayed from then on; the
  * buffers' contents may change between calls.  A lane's workspaces are sized
- * for the largest item it has run.  Output buffers of different items must
- * not overlap. */
+ * for the largest item it has run, and given back when the context itself
+ * finds no room for one.  Output buffers of different items must not
+ * overlap. */
 abs_status abs_estimate_batched(abs_ctx *ctx, int32_t n_items, const abs_item *items);
 
 /* abs_estimate_batched from HOST memory: every item's d_uv and d_vis are host

@@ -285,7 +285,8 @@ void *workspace(abs_ctx *ctx, const char *name, size_t bytes) {
         w.p = nullptr;
         return false;
     };
-    if (!allocate()) return nullptr;
+    // the lanes' workspaces serve concurrency alone: a context short of memory takes them back
+    if (!allocate() && !(release_lane_workspaces(ctx) && allocate())) return nullptr;
     w.bytes = want;
     return w.p;
 }

@@ -1,5 +1,5 @@
 """Ensembles on a device short of memory: a lane without room for its workspaces hands its realisations back and
-gives what it took back to the device."""
+gives what it took back to the device, and a context that finds no room takes its lanes' workspaces back."""
 import numpy as np
 import pytest
 
@@ -69,3 +69,18 @@ def test_lane_without_room(failures):
         assert torch.cuda.mem_get_info(dev)[0] > before - (64 << 20)
         ctx.close()
 
+
+def test_context_takes_its_lanes_workspaces_back():
+    st, dev, small = _case(96)
+    big = Case(192, st, dev)
+    with torch.cuda.stream(st):
+        ctx = absmod.Context(0, st)
+        for _ in range(3):
+            small.check(ctx)
+        ctx.inject_alloc_failures(1)
+        big.check(ctx)      # its first workspace finds no room until the lanes' are freed
+        ctx.inject_alloc_failures(0)
+        for _ in range(3):
+            small.check(ctx)
+            big.check(ctx)
+        ctx.close()
