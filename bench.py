@@ -315,17 +315,47 @@ def ring_census(mask, q, n):
 
 
 def count_route_visits(A, F):
-    """Pair visits of the exact count kernel, which takes the cheaper of its two routes: the
-    direct enumeration of the filled cells, sum over a <= b of floor(F_a / 2) F_b, or the
-    holes route (H = A - F), sum over a <= b of floor(H_a / 2) A_b + 2 floor(F_a / 2) H_b
-    (the full-annulus table it subtracts from is computed once per configuration).  The unit is
-    the plain enumeration: the kernel's holes route halves the one-hole terms and takes the
-    annulus by its symmetric orbits, so a rate in this unit is above its executed one."""
+    """Pair visits of the plain enumeration, the cheaper of two routes: the direct one over the
+    filled cells, sum over a <= b of floor(F_a / 2) F_b, or the holes route (H = A - F) without
+    the lattice's symmetries, sum over a <= b of floor(H_a / 2) A_b + 2 floor(F_a / 2) H_b (the
+    full-annulus table it subtracts from is computed once per configuration)."""
     H = A - F
     tail = lambda v: np.cumsum(v[::-1])[::-1]          # sum over b >= a
     direct = int(np.sum((F // 2) * tail(F)))
     holes = int(np.sum((H // 2) * tail(A) + 2 * (F // 2) * tail(H)))
     return holes if holes < direct else direct
+
+
+def count_kernel_visits(mask, q, n):
+    """Pair visits of the exact count kernel, and the route it takes: direct, sum over a <= b of
+    (F_a / 2) F_b, or holes: pairs of holes, (H_a / 2) H_b over a <= b against each of two maps,
+    and, for every two rings (a, b), the orbits of ring a that hold a hole (images of a cell under
+    the square's reflections) with the upper-half cells of ring b above half the lowest of them.
+    The kernel picks the route by the same sums with every upper-half cell in place of the last."""
+    A, F = ring_census(mask, q, n)
+    H, nb = A - F, len(q) - 1
+    tail = lambda v: np.cumsum(v[::-1])[::-1]
+    R = max(max(ring_rmax(q, n // 2 - 1)), 0)
+    k = np.arange(-R, R + 1)
+    y, x = np.meshgrid(np.arange(R + 1), k, indexing="ij")       # upper half plane, row-major
+    r2 = x.astype(np.int64) ** 2 + y.astype(np.int64) ** 2
+    on = ((y > 0) | (x > 0)) & (r2 >= q[0]) & (r2 < q[-1])
+    x, y = x[on], y[on]
+    ring = np.searchsorted(np.asarray(q), r2[on], side="right") - 1
+    key = y.astype(np.int64) * (2 * (3 * R + 1)) + x
+    hole = mask[y % n, x % n] == 0
+    lo, hi = np.minimum(np.abs(x), np.abs(y)), np.maximum(np.abs(x), np.abs(y))
+    held = np.unique((hi.astype(np.int64) * (R + 1) + lo)[hole])       # orbits with holes, by their (y, x) = (hi, lo)
+    hy, hx = held // (R + 1), held % (R + 1)
+    orbits = np.bincount(np.searchsorted(np.asarray(q), hx ** 2 + hy ** 2, side="right") - 1, minlength=nb)[:nb]
+    direct = int(np.sum((F // 2) * tail(F)))
+    pairs = int(np.sum((H // 2) * tail(H)))
+    if not 2 * pairs + int(orbits.sum()) * len(x) < direct:
+        return direct, "direct"
+    lowest = [key[(ring == a) & (x >= 0) & (x <= y)].min(initial=np.iinfo(np.int64).max) for a in range(nb)]
+    ups = [np.sort(key[ring == b]) for b in range(nb)]
+    one = sum(int(orbits[a]) * sum(int(np.sum(2 * u > lowest[a])) for u in ups) for a in range(nb) if orbits[a])
+    return 2 * pairs + one, "holes"
 
 
 def ring_rmax(q, half):
@@ -421,9 +451,9 @@ def channel_geometry(m, cfg, ctx, items, torch, dev):
     for it in items:
         ctx.abs_grid(cfg, it[1], it[2], g, w, mk)
         ctx.sync()
-        A, F = ring_census(mk.cpu().numpy(), q, n)
-        visits += count_route_visits(A, F)
-        fills += int(F.sum())
+        mask = mk.cpu().numpy()
+        visits += count_kernel_visits(mask, q, n)[0]
+        fills += int(ring_census(mask, q, n)[1].sum())
     N = m.abs_fft_size(cfg)
     k = len(items)
     return {"pair_visits": visits / k, "filled": fills / k, "n_trip": len(m.abs_triplets(cfg)), "P": N * N,
