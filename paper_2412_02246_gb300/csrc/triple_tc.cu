@@ -126,7 +126,7 @@ constexpr int B_ROWS = 8;            // B windows start and end on 8-ring bounda
 #ifndef ABS_TC_DRAIN
 #define ABS_TC_DRAIN 8
 #endif
-constexpr int DRAIN = ABS_TC_DRAIN;  // chunks accumulated in tensor memory before the formers drain them
+constexpr int DRAIN = ABS_TC_DRAIN;  // chunks accumulated in tensor memory before the drainers take them
 #ifndef ABS_TC_SET_COLS
 #define ABS_TC_SET_COLS 128
 #endif
@@ -235,6 +235,15 @@ __device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t count) {
 
 __device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
     asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];\n" ::"r"(mbar) : "memory");
+}
+
+// An arrival of the lanes that are `on`, without a branch: the warp stays together.
+__device__ __forceinline__ void mbar_arrive_if(uint32_t mbar, bool on) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %1, 0;\n\t"
+        "@p mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];\n\t}\n"
+        ::"r"(mbar), "r"((int)on) : "memory");
 }
 
 __device__ __forceinline__ void mbar_arrive_tx(uint32_t mbar, uint32_t bytes) {
@@ -531,7 +540,7 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
                 } else {
                     d_cur += d_stage;
                 }
-                if (gc == DRAIN - 1 || c == nchunks - 1) {   // the group is complete: the formers drain it
+                if (gc == DRAIN - 1 || c == nchunks - 1) {   // the group is complete: the drainers take it
                     mma_commit(smem_u32(&d_full[grp & 1]));
                     ++grp;
                 }
@@ -608,8 +617,7 @@ __global__ void __maxnreg__(TC_MAXREG) k_triple_tc(TcParams G, TcPlanes PL,
                     asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
                     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&a_full[(cg & (ASLOTS - 1)) * MAX_TILES + t]));
-                    __syncwarp();
+                    mbar_arrive_if(smem_u32(&a_full[(cg & (ASLOTS - 1)) * MAX_TILES + t]), lane == 0);
                 }
                 // tiles the set does not have: their barriers keep step with the chunks
                 if (lane == 0)
