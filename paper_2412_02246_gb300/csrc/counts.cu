@@ -29,17 +29,17 @@
 // half plane and u above h/2 (row-major), the self-mapped g2 = -h/2 apart; above
 // h/2, because h + g2 = h - u is then the shorter of the two third vertices'
 // candidates and mostly inside the annuli.  T(A,A,A) is enumerated per orbit as well (every orbit,
-// weighted by its size).  The two-hole terms are enumerated directly, |H|^2 / 4
-// pairs each.  A channel of the wide-band workload (R = 350, 385,000 cells,
-// 33,000 holes in the outer rings) has 2.7e8 visits of the one-hole terms this
-// way and 5e8 of the others, against 1.3e10 for the form
-// T(A,A,A) - T(H,A,A) - T(F,H,A) - T(F,F,H) without the symmetries.  A
+// weighted by its size).  The two-hole terms are enumerated directly, sum over
+// a <= b of |H_a| |H_b| / 2 pairs each.  A channel of the wide-band workload
+// (R = 350, 385,000 cells, 33,000 holes in the two outer rings) has 4.6e8 visits
+// of the one-hole terms this way and 8.4e8 of the others, against 1.2e10 for the
+// form T(A,A,A) - T(H,A,A) - T(F,H,A) - T(F,F,H) without the symmetries.  A
 // device-side estimate picks this route or the direct enumeration of T(F,F,F),
 // whichever visits fewer pairs; both are exact.
 //
 // Cell lists are row-major per ring and hold the upper half plane only (the
 // lower half is the negation).  The lists of A and of the orbits and the byte
-// map of A are geometry, made with the setup.  A byte map holds 1 + ring id of
+// map of A are geometry, made once per configuration at its first count.  A byte map holds 1 + ring id of
 // every cell of a family (0 elsewhere), indexed by |lin(h)| with lin(g) = g_y W +
 // g_x, W = 2R + 1: lin is linear and odd, so lin(g1 + g2) = lin(g1) + lin(g2) and
 // |lin(h)| = lin(+-h) picks the upper-half-plane representative of h, whose

@@ -915,7 +915,7 @@ FftLaunch fft_launch(const Setup &s, int sm_count) {
     // (double-float) a thread
     const int per_sm = std::min(2048 / FFT_NT, 65536 / (FFT_NT * (f32 ? 32 : 64)));
     L.CB = lines_per_cta(line, 2 * s.R + 1, npairs, sm_count, per_sm);
-    L.RB = 2;   // the row pass: see default_rows (the autotuner tries 1 to 8)
+    L.RB = 0;   // the row pass: the caller's default_rows (the autotuner tries 1 to 8)
     L.col_smem = line * 2 * L.CB;   // two line buffers
     return L;
 }

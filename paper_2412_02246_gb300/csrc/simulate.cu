@@ -100,8 +100,10 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
 
 // SIM_V visibilities a thread, SIM_A columns from blockIdx.y SIM_A, rows [blockIdx.z rows_per, + rows_per):
 // their sums over them as double-float pairs (re.hi, re.lo, im.hi, im.lo) in part[z gridDim.y + y][vis].
-// Bound by FP32 multiply-adds: per term one half of a packed FFMA2 for each of re and im; one map load
-// (LDS.128, a broadcast) serves four FFMA2 of each visibility.  The columns' FP32 sums run in chains of
+// Per term one half of a packed FFMA2 (two columns) for each of re and im; one map load (LDS.128, a
+// broadcast) serves four FFMA2 of each visibility.  The columns' phases take 243 registers a thread, so two
+// CTAs an SM: issue 53 %, the FMA pipe 43 %, what is between is the chains' latency (100,000 visibilities of
+// 256^2: 0.60 ms against 0.33 of multiply-adds).  The columns' FP32 sums run in chains of
 // SIM_A / 2 terms, eight rows' terms are added in FP32 and everything beyond in double-float; a row
 // phase is rotated from the one SIM_R rows before, at most SIM_ROWS / SIM_R times from an exact one.
 __global__ void __launch_bounds__(SIM_T) k_dft(int m, double dth, const float *__restrict__ W, int64_t n_vis,

@@ -60,8 +60,8 @@
 // triplet's entry.
 //
 // What bounds it: the formers, eight warps each with a serial chain of loads, products,
-// splits and stores a tile (1.80 ms on 128 rings of 1,080^2, of which the MMAs alone take
-// 0.9; issue 49 %, ALU 43 %, the shared-memory data path 68 %).  Draining in warps of
+// splits and stores a tile (1.82 ms on 128 rings of 1,080^2, of which the MMAs alone take
+// 0.9; half of the issue slots, ALU 43 %, two thirds of the shared-memory data path).  Draining in warps of
 // their own took 0.1 ms off: the long accumulators, 64 registers a thread, had left the
 // formers spilling.
 //
